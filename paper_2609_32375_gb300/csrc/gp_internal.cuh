@@ -403,7 +403,7 @@ struct BoxArgs {
     const void* img;
     int64_t pitch;
     const uint8_t* mask;
-    int W, H, B, Mx, nbox, npad;
+    int W, H, B, Mx, nbox;
     double k;
     int maxiter;
     double* bkg;

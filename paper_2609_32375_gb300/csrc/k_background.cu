@@ -7,9 +7,9 @@
 //                  The k-sigma clip then runs on the histogram, not on the
 //                  pixels: each pass is two range sums and one or two order
 //                  statistics, all in exact integer arithmetic.
-//  k_boxstats_f32  one CTA per box (<= 16,384 pixels): values sorted in
-//                  shared memory (bitonic), the clipped set is an index range
-//                  of the sorted array, sums in compensated FP32.
+//  k_boxstats_f32  one CTA per box (<= 16,384 pixels): values in registers,
+//                  the clipped set is a range of values, its median from
+//                  histograms of the range, sums in compensated FP32.
 //  k_mesh_finalize fills boxes with < 50 % good pixels from valid neighbours
 //                  and median-filters both meshes (one CTA, tiny).
 //  k_spline_*      second-derivative tables of the tensor-product natural
@@ -18,6 +18,7 @@
 #include <float.h>
 #include <math.h>
 
+#include "block_select.cuh"
 #include "gp_internal.cuh"
 #include "gp_launch.h"
 
@@ -174,9 +175,13 @@ __device__ __forceinline__ void clip_histogram(Q& q, uint32_t vmin, uint32_t vma
 }
 
 // rank of quantile q of n good values (features for the learned background)
+// : floor(q (n - 1) + 1/2) with q = mantissa 2^-e, exact in integers (and
+// without this GPU's slow float64)
 __device__ __forceinline__ unsigned long long quantile_rank(float q, uint32_t n)
 {
-    return (unsigned long long)floor((double)q * (double)(n - 1) + 0.5);
+    const uint32_t u = __float_as_uint(q);
+    const int e = 150 - (int)(u >> 23);
+    return ((unsigned long long)((u & 0x7fffffu) | 0x800000u) * (n - 1u) + (1ull << (e - 1))) >> e;
 }
 
 __device__ void boxstats_u16_box(const BoxArgs& A, int box, uint32_t* hist);
@@ -747,130 +752,498 @@ __global__ void __launch_bounds__(WB_NT, 8) k_boxstats_win(const BoxArgs* __rest
 }
 
 // ============================================================ float32 box ===
-constexpr int F32_NT = 512;
+// One CTA per box, its values in registers (VPT a thread, NaN where bad or
+// clipped away: no range test accepts those).  A clip pass needs the count,
+// the sums and the median of the values in a range, so nothing is sorted: a
+// histogram of the range, kept as prefix counts, names the few values among
+// which the median lies, and later passes (their ranges are nested) use the
+// same histogram until their range is an eighth of its own.
+//   each pass: values out of range dropped, count and sum  | barrier
+//              warp 0: mean; the median's bin              | barrier
+//              squared deviations; that bin's values       | barrier
+//              warp 0: sigma, median, next range           | barrier
+// Bound by instruction issue and the barriers' latency: 32 us for the 256 boxes
+// of a 1 MP frame at mesh 64 and 106 us for a masked 9 MP one, where a bitonic
+// sort of each box (78 block-wide steps of 4,096 values) took 183 and 721; the
+// quantiles of a 17 MP frame take 91 us against 523.  Two float32 values take one paired operation
+// in the compensated sums, and mean, sigma and range are float-float too, on
+// one warp: this GPU issues a float64 warp instruction every 16 cycles an SM,
+// and its long latency sits in the chain of every pass.
+constexpr int F32_LIST = 64;      // values among which the median is ranked
 
-__device__ __forceinline__ DF block_df_sum(DF v, DF* red)
+__device__ __forceinline__ unsigned long long f2pack(float a, float b)
 {
-    v = df_warp_sum(v);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    __syncthreads();
-    if (lane == 0) red[warp] = v;
-    __syncthreads();
-    DF t = lane < (int)(blockDim.x >> 5) ? red[lane] : df_zero();
-    t = df_warp_sum(t);
-    return t;
+    return (unsigned long long)__float_as_uint(a) | ((unsigned long long)__float_as_uint(b) << 32);
+}
+__device__ __forceinline__ float f2lo(unsigned long long a) { return __uint_as_float((uint32_t)a); }
+__device__ __forceinline__ float f2hi(unsigned long long a) { return __uint_as_float((uint32_t)(a >> 32)); }
+__device__ __forceinline__ unsigned long long f2add(unsigned long long a, unsigned long long b)
+{
+    unsigned long long d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ unsigned long long f2sub(unsigned long long a, unsigned long long b)
+{
+    unsigned long long d;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ unsigned long long f2mul(unsigned long long a, unsigned long long b)
+{
+    unsigned long long d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ unsigned long long f2fma(unsigned long long a, unsigned long long b, unsigned long long c)
+{
+    unsigned long long d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
 }
 
-// first index in [lo, hi) with (double)v[i] >= x (v ascending)
-__device__ __forceinline__ int lower_bound_d(const float* v, int lo, int hi, double x)
+// two float-float accumulators side by side (df_add for each)
+struct DF2 {
+    unsigned long long hi, lo;
+};
+__device__ __forceinline__ void df2_add(DF2& s, unsigned long long v)
 {
-    while (lo < hi) {
-        int mid = (lo + hi) >> 1;
-        if ((double)v[mid] < x) lo = mid + 1; else hi = mid;
+    const unsigned long long t = f2add(s.hi, v);
+    const unsigned long long bp = f2sub(t, s.hi);
+    const unsigned long long e = f2add(f2sub(s.hi, f2sub(t, bp)), f2sub(v, bp));
+    s.hi = t;
+    s.lo = f2add(s.lo, e);
+}
+__device__ __forceinline__ DF df2_sum(const DF2& s)
+{
+    DF a, b;
+    a.hi = f2lo(s.hi); a.lo = f2lo(s.lo);
+    b.hi = f2hi(s.hi); b.lo = f2hi(s.lo);
+    return df_merge(a, b);
+}
+
+template <int NT>
+struct F32Box {
+    __align__(16) uint32_t pre[SEL_BPT * NT + 4];     // values in the bins before; [NB] the total
+    __align__(16) SelShared<NT> sel;
+    uint32_t wsum[NT / 32];
+    DF red[NT / 32];
+    uint32_t cnt[NT / 32];                // kept | dropped below << 16
+    uint32_t kmin, kmax;
+    uint32_t list[5][F32_LIST], nlist[5];
+    // what warp 0 tells the others
+    float mh, ml, flo, fhi;               // the mean (high, low part); the kept range
+    float blo, bhi;                       // range of the values to rank
+    uint32_t m, r;                        // how many they are; the (lower) median's rank among them
+    int rebuild;
+    uint32_t qbin[5], qm[5], qr[5];
+    uint32_t flag[SEL_BPT * NT / 32];     // a bit per bin: holds a quantile
+};
+
+// float-float helpers: |a| >= |b| in df_fast; quotients and roots are a float
+// estimate and one correction from the exact residual (about 46 bits)
+__device__ __forceinline__ DF df_fast(float a, float b)
+{
+    DF r;
+    r.hi = a + b;
+    r.lo = b - (r.hi - a);
+    return r;
+}
+__device__ __forceinline__ DF df_div(DF a, float n)
+{
+    const float q = a.hi / n;
+    const float r = fmaf(-q, n, a.hi) + a.lo;
+    return df_fast(q, r / n);
+}
+__device__ __forceinline__ DF df_sqrt(DF a)
+{
+    if (!(a.hi > 0.f)) return df_zero();
+    const float s = sqrtf(a.hi);
+    return df_fast(s, (fmaf(-s, s, a.hi) + a.lo) / (2.f * s));
+}
+// the smallest float >= a (sign = 1), the largest <= a (sign = -1)
+__device__ __forceinline__ float df_bound(DF a, float sign)
+{
+    return a.lo * sign > 0.f ? nextafterf(a.hi, sign * INFINITY) : a.hi;
+}
+// med + f sd
+__device__ __forceinline__ DF df_step(DF med, float f, DF sd)
+{
+    DF r = med;
+    df_add_prod(r, f, sd.hi);
+    r.lo = fmaf(f, sd.lo, r.lo);
+    return df_fast(r.hi, r.lo);
+}
+// sum over the first NW lanes (a power of two), in lane 0 .. NW - 1
+template <int NW>
+__device__ __forceinline__ DF df_sum_lanes(DF v)
+{
+#pragma unroll
+    for (int o = NW / 2; o > 0; o >>= 1) {
+        DF w;
+        w.hi = __shfl_xor_sync(0xffffffffu, v.hi, o);
+        w.lo = __shfl_xor_sync(0xffffffffu, v.lo, o);
+        v = df_merge(v, w);
     }
-    return lo;
+    return v;
 }
 
-// first index in [lo, hi) with (double)v[i] > x
-__device__ __forceinline__ int upper_bound_d(const float* v, int lo, int hi, double x)
+// histogram of the keys in [klo, khi], as prefix counts
+template <int NT, class Each>
+__device__ __forceinline__ void box_histogram(Each each, uint32_t klo, int shift, F32Box<NT>& S)
 {
-    while (lo < hi) {
-        int mid = (lo + hi) >> 1;
-        if ((double)v[mid] <= x) lo = mid + 1; else hi = mid;
+    constexpr int NB = SEL_BPT * NT;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    for (int b = tid; b < NB / 4; b += NT) reinterpret_cast<uint4*>(S.pre)[b] = make_uint4(0u, 0u, 0u, 0u);
+    __syncthreads();
+    each([&](uint32_t k) { atomicAdd(&S.pre[(k - klo) >> shift], 1u); });
+    __syncthreads();
+    uint32_t c[SEL_BPT], tot = 0;
+#pragma unroll
+    for (int q = 0; q < SEL_BPT / 4; ++q) {
+        const uint4 h = reinterpret_cast<const uint4*>(S.pre)[tid * (SEL_BPT / 4) + q];
+        c[4 * q] = h.x; c[4 * q + 1] = h.y; c[4 * q + 2] = h.z; c[4 * q + 3] = h.w;
+        tot += h.x + h.y + h.z + h.w;
     }
-    return lo;
+    uint32_t incl = tot;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += t;
+    }
+    if (lane == 31) S.wsum[warp] = incl;
+    __syncthreads();
+    uint32_t e = incl - tot;
+#pragma unroll
+    for (int w = 0; w < NT / 32; ++w) e += w < warp ? S.wsum[w] : 0u;
+    uint32_t o[SEL_BPT];
+#pragma unroll
+    for (int q = 0; q < SEL_BPT; ++q) {
+        o[q] = e;
+        e += c[q];
+    }
+#pragma unroll
+    for (int q = 0; q < SEL_BPT / 4; ++q)
+        reinterpret_cast<uint4*>(S.pre)[tid * (SEL_BPT / 4) + q] = make_uint4(o[4 * q], o[4 * q + 1], o[4 * q + 2],
+                                                                              o[4 * q + 3]);
+    if (tid == NT - 1) S.pre[NB] = e;
+    __syncthreads();
 }
 
-__global__ void __launch_bounds__(F32_NT) k_boxstats_f32(const BoxArgs* __restrict__ batch, const __grid_constant__ BoxArgs one)
+// the bin that holds rank r: the last one with at most r values before it (one full warp)
+template <int NT>
+__device__ __forceinline__ int find_bin(const F32Box<NT>& S, uint32_t r)
 {
+    constexpr int NB = SEL_BPT * NT, ST = NB / 32;
+    const int lane = threadIdx.x & 31;
+    const int top = 31 - __clz(__ballot_sync(0xffffffffu, S.pre[lane * ST] <= r));
+    int best = 0;
+#pragma unroll
+    for (int q = 0; q < ST / 32; ++q) {
+        const unsigned m = __ballot_sync(0xffffffffu, S.pre[top * ST + q * 32 + lane] <= r);
+        if (m) best = q * 32 + 31 - __clz(m);
+    }
+    return top * ST + best;
+}
+
+// ranks r and r1 (r or r + 1) of the n values list[0..n) (one full warp; n <= F32_LIST)
+__device__ __forceinline__ void rank_list(const uint32_t* list, uint32_t n, uint32_t r, uint32_t r1, uint32_t* k0,
+                                          uint32_t* k1)
+{
+    const int lane = threadIdx.x & 31;
+    const uint32_t a = lane < n ? list[lane] : 0xffffffffu, b = lane + 32 < n ? list[lane + 32] : 0xffffffffu;
+    uint32_t ra = 0, rb = 0;
+    for (uint32_t j = 0; j < n; ++j) {
+        const uint32_t v = list[j];
+        ra += v < a || (v == a && j < (uint32_t)lane);
+        rb += v < b || (v == b && j < (uint32_t)lane + 32);
+    }
+    const bool ha = lane < n, hb = lane + 32 < n;
+    // exactly one lane holds each rank
+    *k0 = __reduce_max_sync(0xffffffffu, ha && ra == r ? a : hb && rb == r ? b : 0u);
+    *k1 = __reduce_max_sync(0xffffffffu, ha && ra == r1 ? a : hb && rb == r1 ? b : 0u);
+}
+
+__device__ __forceinline__ int range_shift(uint32_t klo, uint32_t khi, int lb)
+{
+    const int bits = 32 - __clz(khi - klo);
+    return bits > lb ? bits - lb : 0;
+}
+
+template <int NT, int VPT, bool QUANT>
+__global__ void __launch_bounds__(NT, 1024 / NT) k_boxstats_f32(const BoxArgs* __restrict__ batch,
+                                                     const __grid_constant__ BoxArgs one)
+{
+    pdl_wait();
+    pdl_release();
+    constexpr int NB = SEL_BPT * NT, NW = NT / 32;
+    constexpr int LB = NB == 4096 ? 12 : NB == 2048 ? 11 : 10;
+    static_assert(NB == 1 << LB && NW >= 4 && VPT % 2 == 0, "layout");
     const BoxArgs& A = frame_args(batch, one);
     if ((int)blockIdx.x >= A.nbox) return;
     const float* __restrict__ img = static_cast<const float*>(A.img);
     const int64_t pitch = A.pitch;
     const uint8_t* __restrict__ mask = A.mask;
-    const int W = A.W, H = A.H, B = A.B, Mx = A.Mx, nbox = A.nbox, npad = A.npad;
+    const int W = A.W, H = A.H, B = A.B, Mx = A.Mx, nbox = A.nbox;
     const double k = A.k;
     const int maxiter = A.maxiter;
-    double* __restrict__ bkg_out = A.bkg;
-    double* __restrict__ rms_out = A.rms;
-    int* __restrict__ valid_out = A.valid;
-    float* __restrict__ quant_out = A.quant;
-    extern __shared__ float vals[];                 // npad
-    __shared__ int ngood_s;
-    __shared__ DF red[32];
+    __shared__ __align__(16) F32Box<NT> S;
     const int box = blockIdx.x;
     const int bi = box % Mx, bj = box / Mx;
     const int x0 = bi * B, x1 = min(x0 + B, W);
     const int y0 = bj * B, y1 = min(y0 + B, H);
-    const int bw = x1 - x0, bh = y1 - y0;
-    const int tid = threadIdx.x;
-    if (tid == 0) ngood_s = 0;
+    const int bw = x1 - x0, np = bw * (y1 - y0);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (tid == 0) { S.kmin = 0xffffffffu; S.kmax = 0u; }
     __syncthreads();
-    for (int p = tid; p < bw * bh; p += F32_NT) {
-        int y = y0 + p / bw, x = x0 + p % bw;
-        float v = __ldg(img + (int64_t)y * pitch + x);
-        bool bad = !isfinite(v) || (mask && mask[(int64_t)y * W + x]);
-        if (!bad) vals[atomicAdd(&ngood_s, 1)] = v;
+    float v[VPT];
+    const int dy = NT / bw, dx = NT - dy * bw;
+    {
+        const int y = tid / bw, xs = tid - y * bw;
+        const float* p = img + (int64_t)(y0 + y) * pitch + x0 + xs;
+        const int64_t step = dy * pitch + dx, wrap = pitch - bw;
+        int x = xs;
+#pragma unroll
+        for (int q = 0; q < VPT; ++q) {
+            v[q] = tid + q * NT < np ? __ldg(p) : NAN;
+            p += step;
+            x += dx;
+            if (x >= bw) { x -= bw; p += wrap; }
+        }
+        if (mask) {
+            const uint8_t* pm = mask + (int64_t)(y0 + y) * W + x0 + xs;
+            const int64_t mstep = (int64_t)dy * W + dx, mwrap = W - bw;
+            uint8_t b[VPT];
+            x = xs;
+#pragma unroll
+            for (int q = 0; q < VPT; ++q) {
+                b[q] = tid + q * NT < np ? __ldg(pm) : 0;
+                pm += mstep;
+                x += dx;
+                if (x >= bw) { x -= bw; pm += mwrap; }
+            }
+#pragma unroll
+            for (int q = 0; q < VPT; ++q)
+                if (b[q]) v[q] = NAN;
+        }
+#pragma unroll
+        for (int q = 0; q < VPT; ++q) v[q] = fabsf(v[q]) < INFINITY ? v[q] : NAN;
+    }
+    auto each = [&](auto f) {
+#pragma unroll
+        for (int q = 0; q < VPT; ++q)
+            if (v[q] == v[q]) f(key_of(v[q]));
+    };
+    uint32_t ng = 0, klo = 0xffffffffu, khi = 0u;
+    each([&](uint32_t key) {
+        ++ng;
+        klo = min(klo, key);
+        khi = max(khi, key);
+    });
+    ng = __reduce_add_sync(0xffffffffu, ng);
+    klo = __reduce_min_sync(0xffffffffu, klo);
+    khi = __reduce_max_sync(0xffffffffu, khi);
+    if (lane == 0) {
+        atomicMin(&S.kmin, klo);
+        atomicMax(&S.kmax, khi);
+        S.cnt[warp] = ng;
     }
     __syncthreads();
-    const int ng = ngood_s;
-    for (int p = ng + tid; p < npad; p += F32_NT) vals[p] = INFINITY;
+    ng = 0;
+#pragma unroll
+    for (int w = 0; w < NW; ++w) ng += S.cnt[w];
+    klo = S.kmin;
+    khi = S.kmax;
     __syncthreads();
-    // bitonic sort, ascending
-    for (int size = 2; size <= npad; size <<= 1)
-        for (int stride = size >> 1; stride > 0; stride >>= 1) {
-            for (int i = tid; i < npad / 2; i += F32_NT) {
-                int lo = 2 * i - (i & (stride - 1));
-                int hi = lo + stride;
-                bool up = ((lo & size) == 0);
-                float a = vals[lo], b = vals[hi];
-                if ((a > b) == up) { vals[lo] = b; vals[hi] = a; }
-            }
-            __syncthreads();
-        }
-    const bool valid = ng > 0 && 2 * ng >= bw * bh;
+    const bool valid = ng > 0 && 2 * ng >= (uint32_t)np;
     if (ng == 0) {
-        if (tid == 0) { bkg_out[box] = 0; rms_out[box] = 0; valid_out[box] = 0; }
-        if (quant_out && tid < 5) quant_out[(int64_t)tid * nbox + box] = 0.f;
+        if (tid == 0) { A.bkg[box] = 0; A.rms[box] = 0; A.valid[box] = 0; }
+        if (QUANT && tid < 5) A.quant[(int64_t)tid * nbox + box] = 0.f;
         return;
     }
-    int lo = 0, hi = ng;
-    double med = 0, mean = 0, sd = 0;
-    for (int it = 0;; ++it) {
-        int n = hi - lo;
-        med = (n & 1) ? (double)vals[lo + n / 2] : 0.5 * ((double)vals[lo + n / 2 - 1] + (double)vals[lo + n / 2]);
-        DF s = df_zero();
-        for (int i = lo + tid; i < hi; i += F32_NT) df_add(s, vals[i]);
-        s = block_df_sum(s, red);
-        double S = df_value(s);
-        mean = S / (double)n;
-        float mh = (float)mean;
-        float ml = (float)(mean - (double)mh);
-        DF q = df_zero();
-        for (int i = lo + tid; i < hi; i += F32_NT) {
-            float d = (vals[i] - mh) - ml;
-            df_add_prod(q, d, d);
+    int shift = range_shift(klo, khi, LB);
+    box_histogram<NT>(each, klo, shift, S);
+
+    if constexpr (QUANT) {
+        // the learned background's features; nothing reads the clipped statistics then
+        const float qs[5] = {0.10f, 0.25f, 0.50f, 0.75f, 0.90f};
+        // once more over the bins from the 10 % to the 90 % point, which outliers made wide
+        uint32_t below = 0;
+        {
+            const uint32_t b0 = find_bin<NT>(S, (uint32_t)quantile_rank(qs[0], ng));
+            const uint32_t b1 = find_bin<NT>(S, (uint32_t)quantile_rank(qs[4], ng));
+            if (shift > 0 && b1 - b0 < NB / 4) {
+                below = S.pre[b0];
+                const uint32_t top = klo + (b1 << shift) + ((1u << shift) - 1u);
+                khi = min(khi, top);
+                klo += b0 << shift;
+                shift = range_shift(klo, khi, LB);
+                __syncthreads();
+                box_histogram<NT>([&](auto f) {
+                    each([&](uint32_t key) { if (key >= klo && key <= khi) f(key); });
+                }, klo, shift, S);
+            }
         }
-        q = block_df_sum(q, red);
-        sd = sqrt(fmax(df_value(q), 0.0) / (double)n);
+        if (warp == 0) {
+            for (int i = lane; i < NB / 32; i += 32) S.flag[i] = 0u;
+            __syncwarp();
+            for (int q = 0; q < 5; ++q) {
+                const uint32_t r = (uint32_t)quantile_rank(qs[q], ng) - below, b = find_bin<NT>(S, r);
+                if (lane == 0) {
+                    S.qbin[q] = b;
+                    S.qm[q] = S.pre[b + 1] - S.pre[b];
+                    S.qr[q] = r - S.pre[b];
+                    S.nlist[q] = 0;
+                    S.flag[b >> 5] |= 1u << (b & 31);
+                }
+            }
+        }
+        __syncthreads();
+        // the few values of those bins, each into the lists of its quantiles
+        each([&](uint32_t key) {
+            if (key < klo || key > khi) return;
+            const uint32_t b = (key - klo) >> shift;
+            if (!((S.flag[b >> 5] >> (b & 31)) & 1u)) return;
+            for (int q = 0; q < 5; ++q)
+                if (S.qbin[q] == b) {
+                    const uint32_t i = atomicAdd(&S.nlist[q], 1u);
+                    if (i < F32_LIST) S.list[q][i] = key;
+                }
+        });
+        __syncthreads();
+        for (int q = warp; q < 5; q += NW)
+            if (S.qm[q] <= F32_LIST) {
+                uint32_t k0, k1;
+                rank_list(S.list[q], S.qm[q], S.qr[q], S.qr[q], &k0, &k1);
+                if (lane == 0) A.quant[(int64_t)q * nbox + box] = key_value(k0);
+            }
+        for (int q = 0; q < 5; ++q)
+            if (S.qm[q] > F32_LIST) {             // many equal or close values
+                const uint32_t lo = klo + (S.qbin[q] << shift);
+                const uint32_t key = block_select<NT>(each, lo, min(khi, lo + ((1u << shift) - 1u)), S.qr[q], nullptr,
+                                                      S.sel);
+                if (tid == 0) A.quant[(int64_t)q * nbox + box] = key_value(key);
+            }
+        if (tid == 0) A.valid[box] = valid;
+        return;
+    } else {
+
+    float flo = key_value(klo), fhi = key_value(khi);     // the kept range
+    uint32_t n = 0, below = 0;                            // kept values; those dropped below the range
+    DF med = df_zero(), mean = df_zero(), sd = df_zero();   // (lane 0 of warp 0)
+    const float kf = (float)k;                            // clip_k is a float
+    bool rebuild = false;
+    for (int it = 0;; ++it) {
+        DF2 s2;
+        s2.hi = s2.lo = 0ull;
+        uint32_t c = 0;
+#pragma unroll
+        for (int q = 0; q < VPT; q += 2) {
+            float x[2];
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const bool in = v[q + e] >= flo && v[q + e] <= fhi;
+                c += (v[q + e] < flo ? 65536u : 0u) + (in ? 1u : 0u);
+                x[e] = in ? v[q + e] : 0.f;
+                v[q + e] = in ? v[q + e] : NAN;
+            }
+            df2_add(s2, f2pack(x[0], x[1]));
+        }
+        DF s = df_sum_lanes<32>(df2_sum(s2));
+        c = __reduce_add_sync(0xffffffffu, c);
+        if (lane == 0) {
+            S.red[warp] = s;
+            S.cnt[warp] = c;
+        }
+        __syncthreads();
+        c = 0;
+#pragma unroll
+        for (int w = 0; w < NW; ++w) c += S.cnt[w];
+        const uint32_t nn = c & 0xffffu;
+        if (it > 0 && (nn == n || nn == 0)) break;        // the kept set did not change (or rounding emptied it)
+        n = nn;
+        below += c >> 16;
+        if (rebuild) {
+            klo = key_of(flo);
+            khi = key_of(fhi);
+            shift = range_shift(klo, khi, LB);
+            box_histogram<NT>(each, klo, shift, S);
+            below = 0;
+        }
+        const uint32_t r0 = below + (n - 1) / 2, r1 = below + n / 2;
+        if (warp == 0) {
+            s = df_sum_lanes<NW>(S.red[lane < NW ? lane : 0]);
+            mean = df_div(df_fast(s.hi, s.lo), (float)n);
+            // the bins from the one with rank r0 to the one with rank r1 (those between are empty)
+            const uint32_t b0 = find_bin<NT>(S, r0), b1 = r1 < S.pre[b0 + 1] ? b0 : find_bin<NT>(S, r1);
+            if (lane == 0) {
+                S.mh = mean.hi;
+                S.ml = mean.lo;
+                // a bin can reach below the kept range: values dropped there still count in its prefix
+                const uint32_t kl = klo + (b0 << shift), kh = klo + (b1 << shift) + ((1u << shift) - 1u);
+                S.blo = key_value(kl);
+                S.bhi = key_value(min(kh, khi));
+                S.m = S.pre[b1 + 1] - S.pre[b0];
+                S.r = S.pre[b0] > below ? r0 - S.pre[b0] : r0 - below;
+                S.nlist[0] = 0;
+            }
+        }
+        __syncthreads();
+        const float mh = S.mh, ml = S.ml;
+        const float blo = fmaxf(S.blo, flo), bhi = fminf(S.bhi, fhi);
+        const bool listed = S.m <= F32_LIST;
+        const unsigned long long mh2 = f2pack(mh, mh), ml2 = f2pack(ml, ml);
+        s2.hi = s2.lo = 0ull;
+#pragma unroll
+        for (int q = 0; q < VPT; q += 2) {
+            const unsigned long long d = f2sub(f2sub(f2pack(v[q], v[q + 1]), mh2), ml2);
+            const float d0 = v[q] == v[q] ? f2lo(d) : 0.f, d1 = v[q + 1] == v[q + 1] ? f2hi(d) : 0.f;
+            const unsigned long long dd = f2pack(d0, d1), p = f2mul(dd, dd);
+            const unsigned long long np2 = p ^ 0x8000000080000000ull;
+            df2_add(s2, p);
+            s2.lo = f2add(s2.lo, f2fma(dd, dd, np2));
+#pragma unroll
+            for (int e = 0; e < 2; ++e)
+                if (listed && v[q + e] >= blo && v[q + e] <= bhi) {
+                    const uint32_t i = atomicAdd(&S.nlist[0], 1u);
+                    if (i < F32_LIST) S.list[0][i] = key_of(v[q + e]);
+                }
+        }
+        s = df_sum_lanes<32>(df2_sum(s2));
+        if (lane == 0) S.red[warp] = s;
+        __syncthreads();
+        uint32_t k0 = 0, k1 = 0;
+        if (!listed)                                      // many equal or close values
+            k0 = block_select<NT>(each, key_of(blo), key_of(bhi), S.r, r1 > r0 ? &k1 : nullptr, S.sel);
+        if (warp == 0) {
+            s = df_sum_lanes<NW>(S.red[lane < NW ? lane : 0]);
+            sd = df_sqrt(df_div(df_fast(s.hi, s.lo), (float)n));
+            if (listed) rank_list(S.list[0], S.nlist[0], S.r, S.r + (r1 - r0), &k0, &k1);
+            med = df_zero();
+            df_add(med, 0.5f * key_value(k0));
+            df_add(med, 0.5f * key_value(r1 == r0 ? k0 : k1));
+            if (lane == 0) {
+                // values >= med - k sd and <= med + k sd
+                const float nlo = fmaxf(flo, df_bound(df_step(med, -kf, sd), 1.f));
+                const float nhi = fminf(fhi, df_bound(df_step(med, kf, sd), -1.f));
+                S.flo = nlo;
+                S.fhi = nhi;
+                S.rebuild = nlo <= nhi && shift > 0 && (key_of(nhi) - key_of(nlo)) < (khi - klo) / 8;
+            }
+        }
         if (it >= maxiter) break;
-        double flo = med - k * sd, fhi = med + k * sd;
-        int nlo = lower_bound_d(vals, lo, hi, flo);
-        int nhi = upper_bound_d(vals, lo, hi, fhi);
-        if (nhi - nlo == n) break;
-        lo = nlo; hi = nhi;
+        __syncthreads();
+        flo = S.flo;
+        fhi = S.fhi;
+        rebuild = S.rebuild != 0;
     }
     if (tid == 0) {
         double bb, rr;
-        box_result(med, mean, sd, &bb, &rr);
-        bkg_out[box] = valid ? bb : 0.0;
-        rms_out[box] = valid ? rr : 0.0;
-        valid_out[box] = valid;
+        box_result(df_value(med), df_value(mean), df_value(sd), &bb, &rr);
+        A.bkg[box] = valid ? bb : 0.0;
+        A.rms[box] = valid ? rr : 0.0;
+        A.valid[box] = valid;
     }
-    if (quant_out && tid < 5) {
-        const float qs[5] = {0.10f, 0.25f, 0.50f, 0.75f, 0.90f};
-        int r = (int)floor((double)qs[tid] * (double)(ng - 1) + 0.5);
-        quant_out[(int64_t)tid * nbox + box] = vals[r];
     }
 }
 
@@ -1325,9 +1698,6 @@ BoxArgs box_args(const Image& im, int B, double k, int maxiter, double* bkg, dou
     a.W = im.W; a.H = im.H; a.B = B;
     a.Mx = (im.W + B - 1) / B;
     a.nbox = a.Mx * ((im.H + B - 1) / B);
-    int npad = 1;
-    while (npad < B * B) npad <<= 1;
-    a.npad = npad;
     a.k = k; a.maxiter = maxiter;
     a.bkg = bkg; a.rms = rms; a.valid = valid; a.quant = quant;
     a.fb_list = nullptr; a.fb_count = nullptr;
@@ -1354,9 +1724,14 @@ cudaError_t launch_boxstats_any(const BoxArgs& one, const BoxArgs* batch, int nf
         cudaFuncSetAttribute(k_boxstats_u16, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         k_boxstats_u16<<<grid, U16_NT, smem, st>>>(batch, one);
     } else {
-        const size_t smem = (size_t)(batch ? 16384 : one.npad) * sizeof(float);
-        cudaFuncSetAttribute(k_boxstats_f32, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        k_boxstats_f32<<<grid, F32_NT, smem, st>>>(batch, one);
+        // threads and values a thread by box area (the frames of a batch share B)
+        const int area = one.B * one.B;
+        auto run = [&](auto kern, auto quant, int nt) {
+            launch_dep(one.quant ? quant : kern, grid, dim3(nt), 0, st, batch, one);
+        };
+        if (area <= 128 * 8) run(k_boxstats_f32<128, 8, false>, k_boxstats_f32<128, 8, true>, 128);
+        else if (area <= 256 * 16) run(k_boxstats_f32<256, 16, false>, k_boxstats_f32<256, 16, true>, 256);
+        else run(k_boxstats_f32<512, 32, false>, k_boxstats_f32<512, 32, true>, 512);
     }
     return cudaGetLastError();
 }
