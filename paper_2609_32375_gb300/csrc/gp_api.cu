@@ -231,7 +231,7 @@ gp_status run_detect(gp_ctx* ctx, Carver& cv, const gp_image* img, const SplineT
     if (p->nnear) GP_CUDA(cudaMemsetAsync(p->nnear, 0, sizeof(int), st));
     const DetectArgs A = detect_args(im, sb, sr, taps, p->kw, p->kh, p->thresh, p->minarea, segmap, p->mask_out,
                                      p->nnear, nullptr, w.D, w.T, w.P, w.C, ctx->dstatus);
-    GP_CUDA(launch_stream_any(A, nullptr, 1, detect_grid(W, H, false), st));
+    GP_CUDA(launch_stream_any(&A, nullptr, 1, st));
     mark(ctx, 3, st);
     GP_CUDA(launch_label_any(A, nullptr, 1, st, ctx->side_made ? &ctx->side : nullptr));
     mark(ctx, 4, st);
@@ -831,7 +831,7 @@ gp_status gp_label_mask(gp_ctx* ctx, const uint8_t* mask, int32_t width, int32_t
     GP_CUDA(cudaMemsetAsync(w.zero, 0, (size_t)w.nzero * sizeof(int), st));
     const DetectArgs A = detect_args(im, none, none, nullptr, 1, 1, 1.f, minarea, segmap, nullptr, nullptr, mask, w.D,
                                      w.T, w.P, w.C, ctx->dstatus);
-    GP_CUDA(launch_stream_any(A, nullptr, 1, detect_grid(width, height, true), st));
+    GP_CUDA(launch_stream_any(&A, nullptr, 1, st));
     mark(ctx, 3, st);
     GP_CUDA(launch_label_any(A, nullptr, 1, st, nullptr));
     mark(ctx, 4, st);

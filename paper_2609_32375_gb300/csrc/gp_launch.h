@@ -25,12 +25,10 @@ cudaError_t launch_bkg_maps(const SplineTab& sb, const SplineTab& sr, int W, int
                             cudaStream_t st);
 
 // detection (k_stream.cu: threshold mask; k_detect.cu: labelling, merge, rank)
-int stream_ctas(int W, int H);
-int pack_warps(int W, int H);
 int stream_ks(int kw, int kh);
-int detect_grid(int W, int H, bool given_mask);
-cudaError_t launch_stream_any(const DetectArgs& one, const DetectArgs* batch, int nframes, int maxgrid,
-                              cudaStream_t st);
+// args: the frames' records on the host (one alone when batch == nullptr, else
+// nframes of them, whose copies batch holds on the device)
+cudaError_t launch_stream_any(const DetectArgs* args, const DetectArgs* batch, int nframes, cudaStream_t st);
 cudaError_t launch_resolve(const Tiles& T, const Pieces& P, const Comps& C, const DetMask& dm, uint32_t* seg, int W,
                            int H, int minarea, int walk_limit, int* status, cudaStream_t st);
 cudaError_t launch_rank(const Comps& C, int* n_out, int capacity, bool place, int* status, cudaStream_t st);

@@ -308,7 +308,7 @@ gp_status run_frames(Exec& ex, int n, FrameIO* F, const Params& P, bool detect)
     std::vector<ResolveArgs> res(detect ? n : 0);
     std::vector<RankArgs> rank(detect ? n : 0);
     std::vector<MeasureArgs> meas(detect ? n : 0);
-    int maxbox = 0, maxgrid = 0, maxtiles = 0;
+    int maxbox = 0, maxtiles = 0;
     size_t mesh_smem = 0;
     for (int f = 0; f < n; ++f) {
         FrameWork& x = w[f];
@@ -336,7 +336,6 @@ gp_status run_frames(Exec& ex, int n, FrameIO* F, const Params& P, bool detect)
         rank[f] = rank_args(x.dw.C, F[f].cat.n, F[f].cat.capacity, true, F[f].status);
         meas[f] = measure_args(im, x.sb, x.sr, x.dw.C, F[f].cat, P.radii, P.nr, P.gain, F[f].apflux, F[f].apferr,
                                F[f].apflags);
-        maxgrid = std::max(maxgrid, detect_grid(x.W, x.H, false));
         maxtiles = std::max(maxtiles, x.dw.T.ntx * x.dw.T.nty);
     }
     const int nfused = (int)mesh.size();
@@ -410,7 +409,7 @@ gp_status run_frames(Exec& ex, int n, FrameIO* F, const Params& P, bool detect)
     // ---- detection, segment resolution, catalog order, measurement
     for (int f = 0; f < n; ++f)
         if (F[f].nnear) PL_CUDA(cudaMemsetAsync(F[f].nnear, 0, sizeof(int), ex.st));
-    PL_CUDA(launch_stream_any(det[0], d_det, n, maxgrid, ex.st));
+    PL_CUDA(launch_stream_any(det.data(), d_det, n, ex.st));
     ex.at(3);
     PL_CUDA(launch_label_any(det[0], d_det, n, ex.st, ex.side));
     ex.at(4);

@@ -1196,7 +1196,6 @@ constexpr int LT_CTAS = 152 * 11;
 constexpr int LT_BIG_CTAS = 152 * 4;
 constexpr int LT_LATE_CTAS = 152;         // the deferred tiles: few or none
 
-int detect_grid(int W, int H, bool given_mask) { return given_mask ? pack_warps(W, H) : stream_ctas(W, H); }
 
 // The crowded tiles: one warp per listed tile counts its foreground pixels
 // from the packed mask (lane = tile row) and lists the tile for the crowded

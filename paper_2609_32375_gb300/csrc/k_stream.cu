@@ -6,14 +6,16 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include <algorithm>
+
 #include "k_stream_impl.cuh"
 
 namespace gp {
 
-cudaError_t launch_stream_u16(const DetectArgs& one, const DetectArgs* batch, int nframes, int maxcta,
-                              const CUtensorMap* map, cudaStream_t st);
-cudaError_t launch_stream_f32(const DetectArgs& one, const DetectArgs* batch, int nframes, int maxcta,
-                              const CUtensorMap* map, cudaStream_t st);
+cudaError_t launch_stream_u16(const DetectArgs& one, const DetectArgs* batch, int nframes, int maxcta, int rows,
+                              bool fast, const CUtensorMap* maps, cudaStream_t st);
+cudaError_t launch_stream_f32(const DetectArgs& one, const DetectArgs* batch, int nframes, int maxcta, int rows,
+                              bool fast, const CUtensorMap* maps, cudaStream_t st);
 
 // ------------------------------------------------------- given masks ---
 // gp_label_mask: the caller's byte mask packed into the same bit layout,
@@ -100,9 +102,7 @@ static bool make_tmap(const Image& im, int G, CUtensorMap* map)
     return r == CUDA_SUCCESS;
 }
 
-int stream_ctas(int W, int H) { return ((W + ST_COLS - 1) / ST_COLS) * ((H + ST_RC - 1) / ST_RC); }
-
-int pack_warps(int W, int H) { return ((W + ST_STRIP - 1) / ST_STRIP) * ((H + TY - 1) / TY); }
+static int pack_warps(int W, int H) { return ((W + ST_STRIP - 1) / ST_STRIP) * ((H + TY - 1) / TY); }
 
 // rows per group of the streaming pass for a padded kernel size
 static int stream_group_rows(int ks)
@@ -122,20 +122,58 @@ int stream_ks(int kw, int kh)
     return k <= 3 ? 3 : k <= 5 ? 5 : k <= 7 ? 7 : 15;
 }
 
-cudaError_t launch_stream_any(const DetectArgs& one, const DetectArgs* batch, int nframes, int maxcta,
-                              cudaStream_t st)
+static int stream_ctas(int W, int H, int rows)
 {
+    return ((W + ST_COLS - 1) / ST_COLS) * ((H + rows - 1) / rows);
+}
+
+// Output rows per CTA.  A CTA takes about as long as its row groups, alone on
+// an SM or with three others there (the most that fit), so the pass lasts its
+// waves of 4 x 152 CTAs times the groups of one, and 1.5 more for filling the
+// pipeline.  Shorter CTAs read and filter more halo rows (8 groups of 5 for
+// 32 rows, 27 for 128).  1 MP float32: 85 us at 128 rows, 33 at 32; 4 MP
+// uint16: 75 and 32; 17 MP float32: 92 and 64 (64 rows).
+static int stream_rows(const DetectArgs* args, int n, int G)
+{
+    int best = ST_RC;
+    double least = 0.0;
+    for (int rows = ST_RC; rows >= TY; rows >>= 1) {
+        int64_t ctas = 0;
+        for (int f = 0; f < n; ++f) ctas += stream_ctas(args[f].im.W, args[f].im.H, rows);
+        const int groups = (rows + 2 * (args[0].ks / 2) + G - 1) / G;
+        const double t = (double)((ctas + 4 * 152 - 1) / (4 * 152)) * (groups + 1.5);
+        if (rows == ST_RC || t < least) {
+            least = t;
+            best = rows;
+        }
+    }
+    return best;
+}
+
+cudaError_t launch_stream_any(const DetectArgs* args, const DetectArgs* batch, int nframes, cudaStream_t st)
+{
+    const DetectArgs& one = args[0];
     if (one.in_mask) {
-        const int blocks = (maxcta + 3) / 4;   // maxcta: pack_warps() of the largest frame
+        int warps = 0;
+        for (int f = 0; f < nframes; ++f) warps = std::max(warps, pack_warps(args[f].im.W, args[f].im.H));
+        const int blocks = (warps + 3) / 4;
         if (batch) k_pack_mask<true><<<dim3(blocks, nframes), 128, 0, st>>>(batch, one);
         else k_pack_mask<false><<<blocks, 128, 0, st>>>(nullptr, one);
         return cudaGetLastError();
     }
-    CUtensorMap map;
-    const bool tma = !batch && make_tmap(one.im, stream_group_rows(one.ks), &map);
-    const CUtensorMap* mp = tma ? &map : nullptr;
-    if (one.im.is_f32) return launch_stream_f32(one, batch, nframes, maxcta, mp, st);
-    return launch_stream_u16(one, batch, nframes, maxcta, mp, st);
+    const int G = stream_group_rows(one.ks), rows = stream_rows(args, nframes, G);
+    CUtensorMap maps[MAX_BATCH];
+    bool fast = one.nrank == 1 && one.ks <= 7, tma = true;
+    int ctas = 0;
+    for (int f = 0; f < nframes; ++f) {
+        const DetectArgs& A = args[f];
+        fast = fast && !A.mask_out && !A.nnear && !A.im.mask;
+        tma = tma && make_tmap(A.im, G, maps + f);
+        ctas = std::max(ctas, stream_ctas(A.im.W, A.im.H, rows));
+    }
+    const CUtensorMap* mp = tma ? maps : nullptr;
+    if (one.im.is_f32) return launch_stream_f32(one, batch, nframes, ctas, rows, fast, mp, st);
+    return launch_stream_u16(one, batch, nframes, ctas, rows, fast, mp, st);
 }
 
 }  // namespace gp

@@ -30,10 +30,22 @@
 //           arrive as zeros and are replaced by their mirror images in the
 //           ring (the border rule of the filter).  Needs 16-byte aligned
 //           rows.
-//   DIRECT  each lane loads its own columns (8- or 16-byte vector loads
-//           where the CTA is inside the frame and rows are aligned, else
-//           element loads at mirrored coordinates), one group ahead in
-//           registers.
+//   DIRECT  the lanes load the warp's columns (8- or 16-byte vector loads of
+//           their own 4 where the CTA is inside the frame and rows are
+//           aligned, else 4 coalesced element loads 32 columns apart, at
+//           mirrored coordinates found once), two groups ahead in registers.
+//           A mask is read in the same way: a masked float becomes NaN in
+//           the stage, a masked uint16 a bit in a register.  A masked 9 MP
+//           float32 frame with unaligned rows takes 118 us (350 with each
+//           element and mask byte loaded, at coordinates mirrored by integer
+//           division, where it was used).
+// Batches whose frames all allow tensor maps use them too: eight 4 MP uint16
+// frames take 96 us (362 in the general direct form).
+//
+// A CTA's rows (a multiple of TY, at most ST_RC) are chosen by the launcher:
+// a group takes about 3 us whatever else the SM runs (a chain of dependent
+// steps within each warp), so a frame that does not fill the SMs with
+// 128-row CTAs is cut into shorter ones (stream_rows).
 // The ring keeps two groups.  The filter pass reads other lanes' columns only
 // in the current group's rows (a warp writes the next group's rows after the
 // barrier that ends every warp's pass over them); the previous group's rows
@@ -54,7 +66,7 @@ constexpr int ST_NT = 32 * ST_NW;
 constexpr int ST_COLS = ST_NW * ST_STRIP;       // 512 columns per CTA
 constexpr int ST_HALO = 8;                      // ring columns each side (>= HMAX, 16-byte multiple)
 constexpr int ST_RW = ST_COLS + 2 * ST_HALO;    // 528 ring columns
-constexpr int ST_RC = 128;                      // output rows per CTA (a multiple of TY)
+constexpr int ST_RC = 128;                      // most output rows per CTA (a multiple of TY)
 constexpr int ST_BOXW = ST_RW / 3;              // 176 columns per TMA box, three boxes per row group
 constexpr int ST_STAGES = 3;                    // TMA stages
 constexpr int ST_WAIT_LIMIT = 1 << 22;          // bounded mbarrier polls (each try_wait also suspends)
@@ -78,8 +90,7 @@ struct StreamSmem {
     static constexpr size_t ring = 0;
     static constexpr size_t ring_bytes = sizeof(float) * 2 * G * ST_RW;
     static constexpr size_t rowc = ring + ring_bytes;
-    static constexpr size_t rowj = rowc + sizeof(float4) * ROWS;
-    static constexpr size_t bar = (rowj + sizeof(int2) * ROWS + 127) & ~(size_t)127;
+    static constexpr size_t bar = (rowc + sizeof(float4) * ROWS + 127) & ~(size_t)127;
     static constexpr size_t stage = bar + 128;
     __host__ __device__ static constexpr size_t box_bytes(int esz) { return ((size_t)ST_BOXW * G * esz + 127) & ~(size_t)127; }
     __host__ __device__ static constexpr size_t total(int esz) { return stage + (size_t)ST_STAGES * 3 * box_bytes(esz); }
@@ -131,47 +142,54 @@ __device__ __forceinline__ void tma_issue(const CUtensorMap* map, uint64_t* bar,
 
 // raw pixels of 4 columns as floats (u16 exact)
 template <bool F32>
+struct PixelType { using T = uint16_t; };
+template <>
+struct PixelType<true> { using T = float; };
+
+template <bool F32>
 struct Raw4;
 template <>
 struct Raw4<false> {
     uint2 w;
+    __device__ __forceinline__ void set(uint16_t a, uint16_t b, uint16_t c, uint16_t d)
+    {
+        w = make_uint2((uint32_t)a | (uint32_t)b << 16, (uint32_t)c | (uint32_t)d << 16);
+    }
+    __device__ __forceinline__ uint16_t get(int e) const
+    {
+        const uint32_t v = e < 2 ? w.x : w.y;
+        return (uint16_t)(e & 1 ? v >> 16 : v);
+    }
     __device__ __forceinline__ void to_float(float* v) const
     {
-        v[0] = (float)(w.x & 0xffffu); v[1] = (float)(w.x >> 16);
-        v[2] = (float)(w.y & 0xffffu); v[3] = (float)(w.y >> 16);
+        // the float 2^23 + u holds a 16-bit u in its low bits: one byte
+        // permutation and one subtraction each, exact, instead of a
+        // conversion on the quarter-rate pipe
+        v[0] = __uint_as_float(__byte_perm(w.x, 0x4b000000u, 0x7610)) - 8388608.f;
+        v[1] = __uint_as_float(__byte_perm(w.x, 0x4b000000u, 0x7632)) - 8388608.f;
+        v[2] = __uint_as_float(__byte_perm(w.y, 0x4b000000u, 0x7610)) - 8388608.f;
+        v[3] = __uint_as_float(__byte_perm(w.y, 0x4b000000u, 0x7632)) - 8388608.f;
     }
 };
 template <>
 struct Raw4<true> {
     float4 w;
+    __device__ __forceinline__ void set(float a, float b, float c, float d) { w = make_float4(a, b, c, d); }
+    __device__ __forceinline__ float get(int e) const { return e == 0 ? w.x : e == 1 ? w.y : e == 2 ? w.z : w.w; }
     __device__ __forceinline__ void to_float(float* v) const { v[0] = w.x; v[1] = w.y; v[2] = w.z; v[3] = w.w; }
 };
 
-// 4 pixels of frame row gy starting at column x (DIRECT): one vector load
-// when `vec`, else element loads at mirrored columns
+// 4 pixels at p (DIRECT, aligned)
 template <bool F32>
-__device__ __forceinline__ Raw4<F32> load4(const Image& im, int gy, int x, bool vec)
+__device__ __forceinline__ Raw4<F32> load4(const void* p)
 {
     Raw4<F32> r;
-    const int64_t row = (int64_t)gy * im.pitch;
-    if (vec) {
-        if constexpr (F32) r.w = __ldg(reinterpret_cast<const float4*>(reinterpret_cast<const float*>(im.data) + row + x));
-        else r.w = __ldg(reinterpret_cast<const uint2*>(reinterpret_cast<const uint16_t*>(im.data) + row + x));
-        return r;
-    }
-    if constexpr (F32) {
-        const float* p = reinterpret_cast<const float*>(im.data) + row;
-        r.w = make_float4(__ldg(p + mirror_idx(x, im.W)), __ldg(p + mirror_idx(x + 1, im.W)),
-                          __ldg(p + mirror_idx(x + 2, im.W)), __ldg(p + mirror_idx(x + 3, im.W)));
-    } else {
-        const uint16_t* p = reinterpret_cast<const uint16_t*>(im.data) + row;
-        r.w = make_uint2((uint32_t)__ldg(p + mirror_idx(x, im.W)) | ((uint32_t)__ldg(p + mirror_idx(x + 1, im.W)) << 16),
-                         (uint32_t)__ldg(p + mirror_idx(x + 2, im.W)) | ((uint32_t)__ldg(p + mirror_idx(x + 3, im.W)) << 16));
-    }
+    if constexpr (F32) r.w = __ldg(reinterpret_cast<const float4*>(p));
+    else r.w = __ldg(reinterpret_cast<const uint2*>(p));
     return r;
 }
 
-// the same 4 pixels from a TMA stage (ring column c, a multiple of 4)
+// 4 pixels of a stage buffer (ring column c, a multiple of 4)
 template <bool F32>
 __device__ __forceinline__ Raw4<F32> stage4(const unsigned char* st, size_t boxb, int s, int c)
 {
@@ -264,22 +282,11 @@ __device__ __forceinline__ float stage1(const unsigned char* st, size_t boxb, in
 
 // one raw pixel into a stage buffer
 template <bool F32>
-__device__ __forceinline__ void stage_put1(unsigned char* st, size_t boxb, int s, int c, float v)
+__device__ __forceinline__ void stage_put1(unsigned char* st, size_t boxb, int s, int c,
+                                           typename PixelType<F32>::T v)
 {
-    constexpr int ESZ = F32 ? 4 : 2;
     const int box = c / ST_BOXW, cc = c - box * ST_BOXW;
-    unsigned char* p = st + box * boxb + ((size_t)s * ST_BOXW + cc) * ESZ;
-    if constexpr (F32) *reinterpret_cast<float*>(p) = v;
-    else *reinterpret_cast<uint16_t*>(p) = (uint16_t)v;
-}
-
-// one pixel of frame row gy at column x (mirrored) as a float (DIRECT)
-template <bool F32>
-__device__ __forceinline__ float load1(const Image& im, int gy, int x)
-{
-    const int64_t i = (int64_t)gy * im.pitch + mirror_idx(x, im.W);
-    if constexpr (F32) return __ldg(reinterpret_cast<const float*>(im.data) + i);
-    else return (float)__ldg(reinterpret_cast<const uint16_t*>(im.data) + i);
+    reinterpret_cast<typename PixelType<F32>::T*>(st + box * boxb)[s * ST_BOXW + cc] = v;
 }
 
 // the spline values of one map at one column x for node rows (j0, j1):
@@ -325,14 +332,23 @@ __device__ __forceinline__ bool bad_at(const Image& im, int x, int y)
 constexpr int SM_DIRECT = 0;   // one frame, lanes load their own columns
 constexpr int SM_TMA = 1;      // one frame, tensor-map copies into shared stages
 constexpr int SM_BATCH = 2;    // a batch of frames (DIRECT loads), grid y = frame
+constexpr int SM_BATCH_TMA = 3;   // a batch of frames, each with its tensor map
+
+// the frames' tensor maps, a kernel parameter (a map in a parameter needs no
+// proxy fence, which one copied to global memory before each call would)
+template <int N>
+struct StreamMaps {
+    CUtensorMap m[N];
+};
+constexpr int stream_nmaps(int mode) { return mode == SM_BATCH_TMA ? MAX_BATCH : 1; }
 
 // FAST: one separable term, no input mask, neither the byte mask nor the
 // near-threshold count requested -- the form the pipeline runs on the
 // workloads; the general form handles the rest.
 template <bool F32, int KS, int MODE, bool FAST>
 __global__ void __launch_bounds__(ST_NT) k_stream(const DetectArgs* __restrict__ batch,
-                                                  const __grid_constant__ DetectArgs one,
-                                                  const __grid_constant__ CUtensorMap tmap)
+                                                  const __grid_constant__ DetectArgs one, int rows,
+                                                  const __grid_constant__ StreamMaps<stream_nmaps(MODE)> maps)
 {
     pdl_wait();
     pdl_release();
@@ -340,7 +356,7 @@ __global__ void __launch_bounds__(ST_NT) k_stream(const DetectArgs* __restrict__
     using SM = StreamSmem<KS>;
     constexpr int H = Cfg::H, G = Cfg::G, NV = Cfg::NV, WOFF = Cfg::WOFF;
     constexpr int ESZ = F32 ? 4 : 2;
-    constexpr bool TMA = MODE == SM_TMA, BATCH = MODE == SM_BATCH;
+    constexpr bool TMA = MODE == SM_TMA || MODE == SM_BATCH_TMA, BATCH = MODE == SM_BATCH || MODE == SM_BATCH_TMA;
     // a pixel can be bad: a non-finite float, or a masked pixel (general form only)
     constexpr bool BADP = F32 || !FAST;
     // bad bits of the main columns, 4 per input row, newest lowest; an
@@ -350,7 +366,6 @@ __global__ void __launch_bounds__(ST_NT) k_stream(const DetectArgs* __restrict__
     extern __shared__ __align__(128) unsigned char smem[];
     float* ring = reinterpret_cast<float*>(smem + SM::ring);
     float4* rowc = reinterpret_cast<float4*>(smem + SM::rowc);
-    int2* rowj = reinterpret_cast<int2*>(smem + SM::rowj);
     uint64_t* bar = reinterpret_cast<uint64_t*>(smem + SM::bar);
     unsigned char* stg = smem + SM::stage;
     constexpr size_t boxb = SM::box_bytes(ESZ);
@@ -359,11 +374,11 @@ __global__ void __launch_bounds__(ST_NT) k_stream(const DetectArgs* __restrict__
     const Image& im = A.im;
     const int W = im.W, Hf = im.H;
     const int ncx = (W + ST_COLS - 1) / ST_COLS;
-    const int ncta = ncx * ((Hf + ST_RC - 1) / ST_RC);
+    const int ncta = ncx * ((Hf + rows - 1) / rows);
     if (BATCH && (int)blockIdx.x >= ncta) return;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int X0 = (blockIdx.x % ncx) * ST_COLS, Y0 = (blockIdx.x / ncx) * ST_RC;
-    const int nout = min(ST_RC, Hf - Y0);
+    const int X0 = (blockIdx.x % ncx) * ST_COLS, Y0 = (blockIdx.x / ncx) * rows;
+    const int nout = min(rows, Hf - Y0);
     const int nin = nout + 2 * H;                         // input rows: frame rows Y0 - H .. Y0 + nout + H - 1
     const int ng = (nin + G - 1) / G;                     // rows past nin are computed (valid addresses) and unused
     const int xs = X0 + ST_STRIP * warp + ST_CPL * lane;  // the lane's first column
@@ -373,11 +388,12 @@ __global__ void __launch_bounds__(ST_NT) k_stream(const DetectArgs* __restrict__
     const int hx = lane < ST_HALO ? X0 - ST_HALO + lane : X0 + ST_COLS + (lane - ST_HALO);
     const int hslot = lane < ST_HALO ? lane : ST_COLS + lane;
 
-    // ---- row table: spline coefficients of every input row (mirrored)
+    const CUtensorMap* tmap = &maps.m[MODE == SM_BATCH_TMA ? blockIdx.y : 0];
+
+    // ---- row table: spline coefficients and node row of every input row (mirrored)
     for (int k = tid; k < ng * G; k += ST_NT) {
         const AxCoef cy = axis_coef(A.sb.ay, (float)mirror_idx(Y0 - H + k, Hf));
-        rowc[k] = make_float4(cy.b, cy.c0, cy.c1, 0.f);
-        rowj[k] = make_int2(cy.i, cy.i1);
+        rowc[k] = make_float4(cy.b, cy.c0, cy.c1, __int_as_float(cy.i));
     }
     if (TMA && tid == 0) {
         for (int s = 0; s < ST_STAGES; ++s)
@@ -386,41 +402,100 @@ __global__ void __launch_bounds__(ST_NT) k_stream(const DetectArgs* __restrict__
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
     constexpr uint32_t gbytes = (uint32_t)(3 * ST_BOXW * G * ESZ);
+    // the node row after node row j (the same one when there is only one)
+    const int jstep = A.sb.ay.n > 1 ? 1 : 0;
     // DIRECT: vector loads when every column of the CTA (and its sides) is
     // inside the frame and rows are aligned; the loads of group g + 2 are in
     // flight during group g's filter pass and land in its stage after it
     const bool vec = !TMA && X0 - ST_HALO >= 0 && X0 + ST_COLS + ST_HALO <= W && (im.pitch % ST_CPL) == 0 &&
                      ((((uintptr_t)im.data) & (F32 ? 15 : 7)) == 0);
+    // columns of the element loads: 32 e + lane of the strip; their mirrored
+    // places in the frame, and the side column's
+    const int ec = ST_STRIP * warp + lane;
+    int mx[4] = {0, 0, 0, 0}, mhx = 0;
+    if (!TMA) {
+#pragma unroll
+        for (int e = 0; e < 4; ++e) mx[e] = vec ? xs + e : mirror_idx(X0 + ec + 32 * e, W);
+        mhx = mirror_idx(hx, W);
+    }
+    const bool masked = !FAST && !TMA && im.mask != nullptr;
     Raw4<F32> raw[G];
-    float hraw[G];
+    typename PixelType<F32>::T hraw[G];
+    // masked uint16 pixels, a bit each (4 per row: the lane's columns), of
+    // the group in work, the next, and the one being fetched; the same for
+    // the side column
+    uint64_t mb0 = 0, mb1 = 0, mb2 = 0;
+    uint32_t hb0 = 0, hb1 = 0, hb2 = 0;
     auto fetch = [&](int g) {
+        using T = typename PixelType<F32>::T;
+        mb2 = 0;
+        hb2 = 0;
 #pragma unroll
         for (int s = 0; s < G; ++s) {
-            const int gy = mirror_idx(Y0 - H + g * G + s, Hf);
-            raw[s] = load4<F32>(im, gy, xs, vec);
-            if (hl) hraw[s] = load1<F32>(im, gy, hx);
+            int gy = Y0 - H + g * G + s;
+            if ((unsigned)gy >= (unsigned)Hf) gy = mirror_idx(gy, Hf);
+            const T* row = reinterpret_cast<const T*>(im.data) + (int64_t)gy * im.pitch;
+            if (vec) raw[s] = load4<F32>(row + xs);
+            else raw[s].set(__ldg(row + mx[0]), __ldg(row + mx[1]), __ldg(row + mx[2]), __ldg(row + mx[3]));
+            if (hl) hraw[s] = __ldg(row + mhx);
+            if (masked) {
+                const uint8_t* mrow = im.mask + (int64_t)gy * W;
+                bool b[4];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) b[e] = __ldg(mrow + mx[e]) != 0;
+                const bool hb = hl && __ldg(mrow + mhx) != 0;
+                if constexpr (F32) {
+                    raw[s].w.x = b[0] ? NAN : raw[s].w.x;
+                    raw[s].w.y = b[1] ? NAN : raw[s].w.y;
+                    raw[s].w.z = b[2] ? NAN : raw[s].w.z;
+                    raw[s].w.w = b[3] ? NAN : raw[s].w.w;
+                    if (hb) hraw[s] = NAN;
+                } else {
+                    uint32_t nib;
+                    if (vec) {
+                        nib = (uint32_t)b[0] | (uint32_t)b[1] << 1 | (uint32_t)b[2] << 2 | (uint32_t)b[3] << 3;
+                    } else {
+                        // the lane's columns 4 lane .. + 3 are bits of the ballot of load lane / 8
+                        const uint32_t w0 = __ballot_sync(0xffffffffu, b[0]), w1 = __ballot_sync(0xffffffffu, b[1]);
+                        const uint32_t w2 = __ballot_sync(0xffffffffu, b[2]), w3 = __ballot_sync(0xffffffffu, b[3]);
+                        const uint32_t wa = lane & 8 ? w1 : w0, wb = lane & 8 ? w3 : w2;
+                        nib = ((lane & 16 ? wb : wa) >> (4 * (lane & 7))) & 15u;
+                    }
+                    mb2 |= (uint64_t)nib << (4 * s);
+                    hb2 |= (uint32_t)hb << s;
+                }
+            }
         }
     };
     auto put = [&](int g) {
         unsigned char* sp = stg + (g % ST_STAGES) * 3 * boxb;
 #pragma unroll
         for (int s = 0; s < G; ++s) {
-            stage_put4<F32>(sp, boxb, s, slot0, raw[s]);
+            if (vec) {
+                stage_put4<F32>(sp, boxb, s, slot0, raw[s]);
+            } else {
+#pragma unroll
+                for (int e = 0; e < 4; ++e) stage_put1<F32>(sp, boxb, s, ST_HALO + ec + 32 * e, raw[s].get(e));
+            }
             if (hl) stage_put1<F32>(sp, boxb, s, hslot, hraw[s]);
         }
     };
     if (!TMA) {
         fetch(0);
         put(0);
+        mb0 = mb2;
+        hb0 = hb2;
         if (ng > 1) {
             fetch(1);
             put(1);
+            mb1 = mb2;
+            hb1 = hb2;
         }
     }
     __syncthreads();
     if (TMA && tid == 0) {
         for (int s = 0; s < ST_STAGES && s < ng; ++s)
-            tma_issue(&tmap, bar + s, stg + s * 3 * boxb, boxb, X0 - ST_HALO, Y0 - H + s * G, gbytes);
+            tma_issue(tmap, bar + s, stg + s * 3 * boxb, boxb, X0 - ST_HALO, Y0 - H + s * G, gbytes);
     }
 
     // per-lane spline state: background at the input rows' node interval
@@ -457,11 +532,11 @@ __global__ void __launch_bounds__(ST_NT) k_stream(const DetectArgs* __restrict__
 #pragma unroll 1
         for (int s = 0; s < G; ++s) {
             const int k = g * G + s;
-            const int2 j = rowj[k];
             const float4 rc = rowc[k];
-            if (j.x != jb) {
-                cb = col4_load(A.sb, j.x, j.y, xs, W, 1.f);
-                jb = j.x;
+            const int j = __float_as_int(rc.w);
+            if (j != jb) {
+                cb = col4_load(A.sb, j, j + jstep, xs, W, 1.f);
+                jb = j;
             }
             float v[4];
             stage4<F32>(sg, boxb, s, slot0).to_float(v);
@@ -473,8 +548,7 @@ __global__ void __launch_bounds__(ST_NT) k_stream(const DetectArgs* __restrict__
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
                     bool b = F32 && !isfinite(v[e]);
-                    if (!FAST && !TMA && im.mask)
-                        b = b || im.mask[(int64_t)mirror_idx(Y0 - H + k, Hf) * W + mirror_idx(xs + e, W)] != 0;
+                    if (!F32 && !FAST && !TMA) b = (mb0 >> (4 * s + e)) & 1u;
                     if (b) m[e] = 0.f;
                     nib |= (uint32_t)b << e;
                 }
@@ -482,14 +556,13 @@ __global__ void __launch_bounds__(ST_NT) k_stream(const DetectArgs* __restrict__
             }
             *reinterpret_cast<float4*>(rg + s * ST_RW + slot0) = make_float4(m[0], m[1], m[2], m[3]);
             if (hl) {
-                if (j.x != jh) {
-                    hcb = col1_load(A.sb, j.x, j.y, hx, W);
-                    jh = j.x;
+                if (j != jh) {
+                    hcb = col1_load(A.sb, j, j + jstep, hx, W);
+                    jh = j;
                 }
                 const float hv = stage1<F32>(sg, boxb, s, hslot);
                 bool b = F32 && !isfinite(hv);
-                if (!FAST && !TMA && im.mask)
-                    b = b || im.mask[(int64_t)mirror_idx(Y0 - H + k, Hf) * W + mirror_idx(hx, W)] != 0;
+                if (!F32 && !FAST && !TMA) b = (hb0 >> s) & 1u;
                 rg[s * ST_RW + hslot] = b ? 0.f : hv - fmaf(rc.z, hcb.w, fmaf(rc.y, hcb.z, fmaf(rc.x, hcb.y, hcb.x)));
             }
         }
@@ -500,7 +573,7 @@ __global__ void __launch_bounds__(ST_NT) k_stream(const DetectArgs* __restrict__
         if (TMA) {
             // the stage is consumed: refill it with group g + S
             if (tid == 0 && g + ST_STAGES < ng)
-                tma_issue(&tmap, bar + g % ST_STAGES, stg + (g % ST_STAGES) * 3 * boxb, boxb, X0 - ST_HALO,
+                tma_issue(tmap, bar + g % ST_STAGES, stg + (g % ST_STAGES) * 3 * boxb, boxb, X0 - ST_HALO,
                           Y0 - H + (g + ST_STAGES) * G, gbytes);
             // columns outside the frame arrived as zeros: mirror images
             if (edge_l || edge_r) {
@@ -588,11 +661,11 @@ __global__ void __launch_bounds__(ST_NT) k_stream(const DetectArgs* __restrict__
             const float F[4] = {acc[(s + 1) % KS][0].x, acc[(s + 1) % KS][0].y, acc[(s + 1) % KS][1].x,
                                 acc[(s + 1) % KS][1].y};
             // k sigma of the output row
-            const int2 jy = rowj[y + H];
             const float4 ry = rowc[y + H];
-            if (jy.x != js) {
-                cs = col4_load(A.sr, jy.x, jy.y, xs, W, A.thresh);
-                js = jy.x;
+            const int jy = __float_as_int(ry.w);
+            if (jy != js) {
+                cs = col4_load(A.sr, jy, jy + jstep, xs, W, A.thresh);
+                js = jy;
             }
             const float2 t01 = col4_eval2(cs, ry, 0), t23 = col4_eval2(cs, ry, 1);
             const float tv4[4] = {t01.x, t01.y, t23.x, t23.y};
@@ -654,7 +727,11 @@ __global__ void __launch_bounds__(ST_NT) k_stream(const DetectArgs* __restrict__
                 }
             }
         }
-        if (!TMA && g + 2 < ng) put(g + 2);
+        if (!TMA) {
+            if (g + 2 < ng) put(g + 2);
+            mb0 = mb1; mb1 = mb2;
+            hb0 = hb1; hb1 = hb2;
+        }
     }
     if (!FAST && A.nnear) {
 #pragma unroll
@@ -664,49 +741,55 @@ __global__ void __launch_bounds__(ST_NT) k_stream(const DetectArgs* __restrict__
 }
 
 template <bool F32, int KS, int MODE, bool FAST>
-cudaError_t launch_stream_inst(const DetectArgs& one, const DetectArgs* batch, int nframes, int maxcta,
-                               const CUtensorMap& map, cudaStream_t st)
+cudaError_t launch_stream_inst(const DetectArgs& one, const DetectArgs* batch, int nframes, int maxcta, int rows,
+                               const CUtensorMap* maps, cudaStream_t st)
 {
     const size_t smem = StreamSmem<KS>::total(F32 ? 4 : 2);
     auto* fn = k_stream<F32, KS, MODE, FAST>;
     cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    launch_dep(fn, dim3(maxcta, nframes), dim3(ST_NT), smem, st, batch, one, map);
+    StreamMaps<stream_nmaps(MODE)> m;
+    memset(&m, 0, sizeof m);
+    if (maps) memcpy(m.m, maps, sizeof(CUtensorMap) * (MODE == SM_BATCH_TMA ? nframes : 1));
+    launch_dep(fn, dim3(maxcta, nframes), dim3(ST_NT), smem, st, batch, one, rows, m);
     return cudaGetLastError();
 }
 
-// the instances of one dtype (k_stream_u16.cu, k_stream_f32.cu)
+// the instances of one dtype (k_stream_u16.cu, k_stream_f32.cu); maps: a
+// tensor map per frame, or null (DIRECT staging)
 template <bool F32>
-cudaError_t launch_stream_dtype(const DetectArgs& one, const DetectArgs* batch, int nframes, int maxcta,
-                                const CUtensorMap* map, cudaStream_t st)
+cudaError_t launch_stream_dtype(const DetectArgs& one, const DetectArgs* batch, int nframes, int maxcta, int rows,
+                                bool fast, const CUtensorMap* maps, cudaStream_t st)
 {
-    const bool fast = one.nrank == 1 && !one.mask_out && !one.nnear && !one.im.mask && one.ks <= 7;
     if (batch) {
-        CUtensorMap m;
-        memset(&m, 0, sizeof m);
+        // FAST batches exist in the TMA form only; the rest take the general direct form
+        if (maps && fast) {
+            switch (one.ks) {
+            case 3: return launch_stream_inst<F32, 3, SM_BATCH_TMA, true>(one, batch, nframes, maxcta, rows, maps, st);
+            case 5: return launch_stream_inst<F32, 5, SM_BATCH_TMA, true>(one, batch, nframes, maxcta, rows, maps, st);
+            case 7: return launch_stream_inst<F32, 7, SM_BATCH_TMA, true>(one, batch, nframes, maxcta, rows, maps, st);
+            default: break;
+            }
+        }
         switch (one.ks) {
-        case 3: return launch_stream_inst<F32, 3, SM_BATCH, false>(one, batch, nframes, maxcta, m, st);
-        case 5: return launch_stream_inst<F32, 5, SM_BATCH, false>(one, batch, nframes, maxcta, m, st);
-        case 7: return launch_stream_inst<F32, 7, SM_BATCH, false>(one, batch, nframes, maxcta, m, st);
-        default: return launch_stream_inst<F32, 15, SM_BATCH, false>(one, batch, nframes, maxcta, m, st);
+        case 3: return launch_stream_inst<F32, 3, SM_BATCH, false>(one, batch, nframes, maxcta, rows, nullptr, st);
+        case 5: return launch_stream_inst<F32, 5, SM_BATCH, false>(one, batch, nframes, maxcta, rows, nullptr, st);
+        case 7: return launch_stream_inst<F32, 7, SM_BATCH, false>(one, batch, nframes, maxcta, rows, nullptr, st);
+        default: return launch_stream_inst<F32, 15, SM_BATCH, false>(one, batch, nframes, maxcta, rows, nullptr, st);
         }
     }
-    const bool tma = map != nullptr;
-    CUtensorMap none;
-    memset(&none, 0, sizeof none);
-    const CUtensorMap& m2 = tma ? *map : none;
 #define GP_STREAM_CASE(KSV)                                                                                       \
     case KSV:                                                                                                     \
-        if (tma) return fast ? launch_stream_inst<F32, KSV, SM_TMA, true>(one, nullptr, 1, maxcta, m2, st)         \
-                             : launch_stream_inst<F32, KSV, SM_TMA, false>(one, nullptr, 1, maxcta, m2, st);       \
-        return fast ? launch_stream_inst<F32, KSV, SM_DIRECT, true>(one, nullptr, 1, maxcta, m2, st)               \
-                    : launch_stream_inst<F32, KSV, SM_DIRECT, false>(one, nullptr, 1, maxcta, m2, st);
+        if (maps) return fast ? launch_stream_inst<F32, KSV, SM_TMA, true>(one, nullptr, 1, maxcta, rows, maps, st)  \
+                              : launch_stream_inst<F32, KSV, SM_TMA, false>(one, nullptr, 1, maxcta, rows, maps, st); \
+        return fast ? launch_stream_inst<F32, KSV, SM_DIRECT, true>(one, nullptr, 1, maxcta, rows, nullptr, st)      \
+                    : launch_stream_inst<F32, KSV, SM_DIRECT, false>(one, nullptr, 1, maxcta, rows, nullptr, st);
     switch (one.ks) {
         GP_STREAM_CASE(3)
         GP_STREAM_CASE(5)
         GP_STREAM_CASE(7)
     default:
-        if (tma) return launch_stream_inst<F32, 15, SM_TMA, false>(one, nullptr, 1, maxcta, m2, st);
-        return launch_stream_inst<F32, 15, SM_DIRECT, false>(one, nullptr, 1, maxcta, m2, st);
+        if (maps) return launch_stream_inst<F32, 15, SM_TMA, false>(one, nullptr, 1, maxcta, rows, maps, st);
+        return launch_stream_inst<F32, 15, SM_DIRECT, false>(one, nullptr, 1, maxcta, rows, nullptr, st);
     }
 #undef GP_STREAM_CASE
 }
