@@ -322,7 +322,7 @@ __device__ __forceinline__ void cr_flags_clean(CrBlock& s, CrMaps& M, const CrAr
 
 // CLEAN: the frame cannot hold a bad pixel (uint16 without a mask); else
 // each CTA looks whether its part does.  17 MP uint16: 804 us with every
-// map computed at every pixel, FIGCR so.
+// map computed at every pixel, 184 us so.
 template <bool F32, bool CLEAN>
 __global__ void __launch_bounds__(CM_NT, CLEAN ? 5 : 2) k_cr(const __grid_constant__ CrArgs A)
 {
