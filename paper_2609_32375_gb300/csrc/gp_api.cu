@@ -621,8 +621,7 @@ gp_status gp_deblend(gp_ctx* ctx, const gp_image* img, const gp_bkg* bkg, const 
     const int rows = cat->capacity > 0 ? cat->capacity : 1;
     DeblendWork w;
     w.cand = cv.take<int>(rows);
-    w.cand_count = cv.take<int>(2);
-    w.obj_count = w.cand_count + 1;
+    w.ctl = cv.take<int>(64);
     w.off = cv.take<int64_t>(rows);
     w.obj_cap = objects->capacity > 0 ? objects->capacity : 1;
     w.obj = cv.take<DbObj>(w.obj_cap);

@@ -72,8 +72,7 @@ struct DbObj {
 };
 struct DeblendWork {
     int* cand;             // [rows] candidate rows
-    int* cand_count;       // [2] candidates, then the staged objects
-    int* obj_count;        // cand_count + 1
+    int* ctl;              // [64] counters (k_deblend.cu)
     int64_t* off;          // [rows] bytes per candidate, then scratch offsets
     DbObj* obj;            // [obj_cap] staged object rows
     int obj_cap;
