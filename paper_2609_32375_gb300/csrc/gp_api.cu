@@ -202,9 +202,9 @@ gp_status run_spline(Carver& cv, const gp_bkg* b, int W, int H, SplineTab* sb, S
                                 st));
         *nlaunch += 1;
     } else {
-        GP_CUDA(launch_spline_tables(b->bkg_mesh, ax, ay, w.scratch, w.tab_b, st));
-        GP_CUDA(launch_spline_tables(b->rms_mesh, ax, ay, w.scratch, w.tab_r, st));
-        *nlaunch += 4;
+        const float* mesh[2] = {b->bkg_mesh, b->rms_mesh};
+        float4* tab[2] = {w.tab_b, w.tab_r};
+        GP_CUDA(launch_spline_tables(mesh, tab, 2, ax, ay, w.scratch, nlaunch, st));
     }
     *sb = make_tab(w.tab_b, W, H, b->mesh);
     *sr = make_tab(w.tab_r, W, H, b->mesh);
@@ -714,12 +714,14 @@ gp_status gp_detect_psf(gp_ctx* ctx, const gp_image* img, const gp_bkg* bkg, con
     carve_det(cv, W, H, cat->capacity, w);
     if (!cv.ok()) return oom(cv);
     const Axis cax = make_axis(W, p->tile), cay = make_axis(H, p->tile);
+    const float* coef[GP_PSF_MAX_MODES];
+    float4* ctab[GP_PSF_MAX_MODES];
     for (int k = 0; k < p->K; ++k) {
-        float4* tab = tabs + (size_t)k * cmx * cmy;
-        GP_CUDA(launch_spline_tables(p->coef + (size_t)k * cmx * cmy, cax, cay, scratch, tab, st));
-        ct[k] = make_tab(tab, W, H, p->tile);
-        ctx->launches += 2;
+        coef[k] = p->coef + (size_t)k * cmx * cmy;
+        ctab[k] = tabs + (size_t)k * cmx * cmy;
+        ct[k] = make_tab(ctab[k], W, H, p->tile);
     }
+    GP_CUDA(launch_spline_tables(coef, ctab, p->K, cax, cay, scratch, &ctx->launches, st));
     mark(ctx, 2, st);
     const Image im = to_image(img);
     GP_CUDA(cudaMemsetAsync(w.zero, 0, (size_t)w.nzero * sizeof(int), st));

@@ -15,7 +15,8 @@ cudaError_t launch_boxstats(const Image& im, int B, double k, int maxiter, doubl
                             float* quant, cudaStream_t st);
 cudaError_t launch_mesh_finalize(double* bkg, double* rms, int* valid, double* tmp_b, double* tmp_r, int* tmp_v,
                                  int Mx, int My, int fsize, float* bkg_out, float* rms_out, cudaStream_t st);
-cudaError_t launch_spline_tables(const float* mesh, Axis ax, Axis ay, double* scratch, float4* tab, cudaStream_t st);
+cudaError_t launch_spline_tables(const float* const* mesh, float4* const* tab, int nmap, Axis ax, Axis ay, double* scratch,
+                                 int* nlaunch, cudaStream_t st);
 size_t spline_scratch_doubles(int Mx, int My);
 bool mesh_fits_smem(int Mx, int My);
 cudaError_t launch_mesh_all(const double* bkg_raw, const double* rms_raw, const int* valid, Axis ax, Axis ay,

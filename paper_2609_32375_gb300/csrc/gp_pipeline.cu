@@ -389,11 +389,11 @@ gp_status run_frames(Exec& ex, int n, FrameIO* F, const Params& P, bool detect)
         if (!learned) {
             PL_CUDA(launch_mesh_finalize(x.bw.bkg_raw, x.bw.rms_raw, x.bw.valid, x.bw.tmp_b, x.bw.tmp_r, x.bw.tmp_v,
                                          x.Mx, x.My, P.bp.filter_size, F[f].bkg.bkg_mesh, F[f].bkg.rms_mesh, ex.st));
-            ex.launches += 1;
+            ex.launches += 2;
         }
-        PL_CUDA(launch_spline_tables(F[f].bkg.bkg_mesh, x.sb.ax, x.sb.ay, x.sw.scratch, x.tab_b, ex.st));
-        PL_CUDA(launch_spline_tables(F[f].bkg.rms_mesh, x.sb.ax, x.sb.ay, x.sw.scratch, x.tab_r, ex.st));
-        ex.launches += 4;
+        const float* mesh[2] = {F[f].bkg.bkg_mesh, F[f].bkg.rms_mesh};
+        float4* tab[2] = {x.tab_b, x.tab_r};
+        PL_CUDA(launch_spline_tables(mesh, tab, 2, x.sb.ax, x.sb.ay, x.sw.scratch, &ex.launches, ex.st));
     }
     for (int f = 0; f < n; ++f) {
         if (!F[f].bkg.bkg_map && !F[f].bkg.rms_map) continue;

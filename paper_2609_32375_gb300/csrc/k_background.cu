@@ -10,10 +10,12 @@
 //  k_boxstats_f32  one CTA per box (<= 16,384 pixels): values in registers,
 //                  the clipped set is a range of values, its median from
 //                  histograms of the range, sums in compensated FP32.
-//  k_mesh_finalize fills boxes with < 50 % good pixels from valid neighbours
-//                  and median-filters both meshes (one CTA, tiny).
-//  k_spline_*      second-derivative tables of the tensor-product natural
-//                  spline through the box centres (FP64 tridiagonal solves).
+//  k_mesh_all      boxes with < 50 % good pixels filled from valid neighbours,
+//                  both meshes median-filtered, second-derivative tables of the
+//                  tensor-product natural spline through the box centres: one
+//                  CTA, for meshes that fit its shared memory.
+//  k_mesh_fill, k_mesh_median, k_spline_lines
+//                  the same for larger meshes (FP64 tridiagonal solves).
 //  k_bkg_maps      optional full-resolution B(p), sigma(p) output.
 #include <float.h>
 #include <math.h>
@@ -1251,26 +1253,30 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_boxstats_f32(const BoxArgs* _
 constexpr int MF_NT = 1024;
 
 // Fill boxes with < 50 % good pixels from the mean of their valid
-// 8-neighbours (sweep after sweep), then median-filter both meshes over a
-// fsize x fsize window clipped at the mesh edge.  One CTA.
+// 8-neighbours (sweep after sweep).  One CTA; most meshes have none to fill
+// and end at the first look.  250 x 251 boxes: 11 us, and 15 for the medians
+// below (1.55 ms when this one CTA copied, sorted and filtered every box).
 __global__ void __launch_bounds__(MF_NT)
-k_mesh_finalize(double* bkg, double* rms, int* valid, double* tmp_b, double* tmp_r, int* tmp_v,
-                int Mx, int My, int fsize, float* bkg_out, float* rms_out)
+k_mesh_fill(double* bkg, double* rms, int* valid, double* tmp_b, double* tmp_r, int* tmp_v, int Mx, int My)
 {
-    __shared__ int missing, any;
+    pdl_wait();
+    pdl_release();
     const int nb = Mx * My, tid = threadIdx.x;
-    if (tid == 0) any = 0;
-    __syncthreads();
-    for (int b = tid; b < nb; b += MF_NT)
-        if (valid[b]) any = 1;
-    __syncthreads();
+    int good = 0, bad = 0;
+#pragma unroll 8
+    for (int b = tid; b < nb; b += MF_NT) {
+        const int v = valid[b];
+        good |= v;
+        bad |= !v;
+    }
+    const bool any = __syncthreads_or(good), some = __syncthreads_or(bad);
+    if (!some) return;
     if (!any) {
         for (int b = tid; b < nb; b += MF_NT) { bkg[b] = 0; rms[b] = 0; valid[b] = 1; }
-        __syncthreads();
+        return;
     }
     for (int sweep = 0; sweep < Mx + My + 2; ++sweep) {
-        if (tid == 0) missing = 0;
-        __syncthreads();
+        bool missing = false;
         for (int b = tid; b < nb; b += MF_NT) {
             tmp_b[b] = bkg[b]; tmp_r[b] = rms[b]; tmp_v[b] = valid[b];
             if (valid[b]) continue;
@@ -1286,104 +1292,182 @@ k_mesh_finalize(double* bkg, double* rms, int* valid, double* tmp_b, double* tmp
                     }
                 }
             if (c) { tmp_b[b] = sb / c; tmp_r[b] = sr / c; tmp_v[b] = 1; }
-            else missing = 1;
+            else missing = true;
         }
-        __syncthreads();
+        const bool more = __syncthreads_or(missing);
         for (int b = tid; b < nb; b += MF_NT) { bkg[b] = tmp_b[b]; rms[b] = tmp_r[b]; valid[b] = tmp_v[b]; }
         __syncthreads();
-        if (!missing) break;
+        if (!more) break;
     }
-    const int h = fsize / 2;
-    for (int b = tid; b < nb; b += MF_NT) {
-        int i = b % Mx, j = b / Mx;
-        for (int map = 0; map < 2; ++map) {
-            const double* src = map ? rms : bkg;
-            double win[49];
-            int c = 0;
-            for (int jj = j - h; jj <= j + h; ++jj)
-                for (int ii = i - h; ii <= i + h; ++ii)
-                    if (ii >= 0 && ii < Mx && jj >= 0 && jj < My) {
-                        double v = src[jj * Mx + ii];
-                        int p = c++;
-                        while (p > 0 && win[p - 1] > v) { win[p] = win[p - 1]; --p; }
-                        win[p] = v;
-                    }
-            double med = (c & 1) ? win[c / 2] : 0.5 * (win[c / 2 - 1] + win[c / 2]);
-            (map ? rms_out : bkg_out)[b] = (float)med;
+}
+
+// Median filter of both meshes over an fsize x fsize window clipped at the
+// mesh edge: a thread per box and map.
+__global__ void __launch_bounds__(256) k_mesh_median(const double* __restrict__ bkg, const double* __restrict__ rms, int Mx,
+                                                     int My, int fsize, float* __restrict__ bkg_out,
+                                                     float* __restrict__ rms_out)
+{
+    pdl_wait();
+    pdl_release();
+    const int nb = Mx * My, t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= 2 * nb) return;
+    const int map = t / nb, b = t - map * nb, i = b % Mx, j = b / Mx;
+    const double* src = map ? rms : bkg;
+    double med;
+    if (fsize == 3) {
+        // the window in registers (absent cells +inf), sorted by odd-even transposition
+        double w[9];
+        int c = 0;
+#pragma unroll
+        for (int k = 0; k < 9; ++k) {
+            const int ii = i - 1 + k % 3, jj = j - 1 + k / 3;
+            const bool in = ii >= 0 && ii < Mx && jj >= 0 && jj < My;
+            w[k] = in ? src[jj * Mx + ii] : (double)INFINITY;
+            c += in ? 1 : 0;
         }
+#pragma unroll
+        for (int pass = 0; pass < 9; ++pass)
+#pragma unroll
+            for (int q = pass & 1; q + 1 < 9; q += 2) {
+                const bool sw = w[q + 1] < w[q];
+                const double lo = sw ? w[q + 1] : w[q], hi = sw ? w[q] : w[q + 1];
+                w[q] = lo;
+                w[q + 1] = hi;
+            }
+        double m0 = w[0], m1 = w[0];
+#pragma unroll
+        for (int q = 1; q < 9; ++q) {
+            if (q == (c - 1) / 2) m0 = w[q];
+            if (q == c / 2) m1 = w[q];
+        }
+        med = (c & 1) ? m1 : 0.5 * (m0 + m1);
+    } else {
+        const int h = fsize / 2;
+        double win[49];
+        int c = 0;
+        for (int jj = j - h; jj <= j + h; ++jj)
+            for (int ii = i - h; ii <= i + h; ++ii)
+                if (ii >= 0 && ii < Mx && jj >= 0 && jj < My) {
+                    double v = src[jj * Mx + ii];
+                    int p = c++;
+                    while (p > 0 && win[p - 1] > v) { win[p] = win[p - 1]; --p; }
+                    win[p] = v;
+                }
+        med = (c & 1) ? win[c / 2] : 0.5 * (win[c / 2 - 1] + win[c / 2]);
     }
+    (map ? rms_out : bkg_out)[b] = (float)med;
 }
 
 // ============================================================ spline tables ===
-// natural-spline second derivatives along a line of n nodes (positions from
-// the axis) for values v (stride vs), written to M (stride ms); d, c are
-// scratch of n doubles.  Thomas algorithm on the interior nodes.
-__device__ void spline_line(const Axis& ax, const double* v, int vs, double* M, int ms, double* c, double* d)
+// Natural-spline second derivatives along lines of n nodes: the tridiagonal
+// system h0 M[r-1] + 2 (h0 + h1) M[r] + h1 M[r+1] = rhs, r = 1 .. n - 2, by
+// elimination and back substitution in float64.  Both recursions forget: the
+// multiplier of what came before is at most about 0.27 a node, so after 32
+// nodes 10^-18 of it is left, and a line is cut into chunks of 64 that start
+// 32 nodes early (and end 32 late) with a zero there.  The pivots, which
+// depend on the node positions only, settle faster still (0.07 a node): each
+// is computed from 24 nodes before it.
+// A CTA takes 32 lines (a lane each) and one chunk of them; its other warps
+// stage.  Bound by the latency of the 224 dependent steps.  A thread per line
+// over the whole line, in global memory, with a division a step took 1.6 ms
+// and 1.1 ms a map for the two passes of a 250 x 251 mesh; both maps together
+// take 57 and 66 us.
+constexpr int SL_CH = 64, SL_OV = 32, SL_N = SL_CH + 2 * SL_OV, SL_NT = 128;
+constexpr int SL_MAPS = 8;
+
+struct SplineMaps {
+    const float* mesh[SL_MAPS];
+    float4* tab[SL_MAPS];
+    double *X[SL_MAPS], *Y[SL_MAPS];
+};
+
+// FINAL = false: X along each mesh row, Y along each mesh column;
+// FINAL = true: XY along each row of Y, then (P, X, Y, XY) as float4.
+// Grid: x the tiles (those of the rows first), y the map.
+template <bool FINAL>
+__global__ void __launch_bounds__(SL_NT) k_spline_lines(const __grid_constant__ SplineMaps maps, Axis ax, Axis ay)
 {
-    const int n = ax.n;
-    for (int i = 0; i < n; ++i) M[i * ms] = 0.0;
-    if (n < 3) return;
-    auto pos = [&](int i) -> double {
-        return (i == n - 1) ? (double)ax.tl : (double)ax.t0 + (double)i * (double)ax.B;
-    };
-    // rows r = 1 .. n-2: h0 M[r-1] + 2 (h0 + h1) M[r] + h1 M[r+1] = rhs
-    double bprev = 0, cprev = 0, dprev = 0;
-    for (int r = 1; r <= n - 2; ++r) {
-        double h0 = pos(r) - pos(r - 1), h1 = pos(r + 1) - pos(r);
-        double a = h0, b = 2.0 * (h0 + h1), cc = h1;
-        double rhs = 6.0 * ((v[(r + 1) * vs] - v[r * vs]) / h1 - (v[r * vs] - v[(r - 1) * vs]) / h0);
-        if (r > 1) {
-            double w = a / bprev;
-            b -= w * cprev;
-            rhs -= w * dprev;
+    pdl_wait();
+    pdl_release();
+    __shared__ double v[SL_N][33];
+    __shared__ double w[SL_N], ib[SL_N], c[SL_N], ih[SL_N + 1];
+    const int Mx = ax.n, My = ay.n, tid = threadIdx.x, lane = tid & 31;
+    const float* mesh = maps.mesh[blockIdx.y];
+    int tile = blockIdx.x;
+    const int rtiles = ((My + 31) / 32) * ((Mx + SL_CH - 1) / SL_CH);
+    const bool rows = FINAL || tile < rtiles;
+    if (!rows) tile -= rtiles;
+    const Axis a = rows ? ax : ay;
+    const int n = a.n, nline = rows ? My : Mx, nch = (n + SL_CH - 1) / SL_CH;
+    const int l0 = tile / nch * 32, c0 = tile % nch * SL_CH, base = c0 - SL_OV;
+    // values of nodes base .. base + SL_N - 1 of the lines
+    for (int q = tid; q < SL_N * 32; q += SL_NT) {
+        const int k = rows ? q % SL_N : q / 32, l = rows ? q / SL_N : q % 32;
+        const int node = base + k, line = l0 + l;
+        double x = 0.0;
+        if (node >= 0 && node < n && line < nline) {
+            const int i = rows ? line * Mx + node : node * Mx + line;
+            x = FINAL ? maps.Y[blockIdx.y][i] : (double)mesh[i];
         }
-        c[r] = cc; d[r] = rhs;
-        bprev = b; cprev = cc; dprev = rhs;
-        M[r * ms] = b;   // keep the pivot temporarily
+        v[k][l] = x;
     }
-    // back substitution
-    double next = 0.0;
-    for (int r = n - 2; r >= 1; --r) {
-        double piv = M[r * ms];
-        double val = (d[r] - c[r] * next) / piv;
-        M[r * ms] = val;
-        next = val;
+    auto pos = [&](int i) -> double { return i == n - 1 ? (double)a.tl : (double)a.t0 + (double)i * (double)a.B; };
+    auto width = [&](int i) -> double { return pos(i + 1) - pos(i); };   // node i to i + 1
+    for (int k = tid; k < SL_N; k += SL_NT) {
+        const int r = base + k;
+        if (r < 1 || r > n - 2) continue;
+        int s = r - 24 > 1 ? r - 24 : 1;
+        double b = 2.0 * (width(s - 1) + width(s)), m = 0.0;
+        for (++s; s <= r; ++s) {
+            const double h0 = width(s - 1);
+            m = h0 / b;
+            b = 2.0 * (h0 + width(s)) - m * h0;
+        }
+        w[k] = m;                 // elimination multiplier (0 for r = 1)
+        ib[k] = 1.0 / b;
+        c[k] = width(r);
+        ih[k] = 1.0 / width(r - 1);
+        ih[k + 1] = 1.0 / width(r);     // the same value as the next thread's
     }
-}
-
-// X: along each mesh row; Y: along each mesh column.  Each of the Mx + My
-// lines has its own scratch line of Mx + My doubles in sc and sd.
-__global__ void k_spline_xy(const float* mesh, Axis ax, Axis ay, double* vals, double* colv, double* X,
-                            double* Y, double* scr_c, double* scr_d)
-{
-    const int Mx = ax.n, My = ay.n;
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t < My) {
-        double* v = vals + (int64_t)t * Mx;
-        for (int i = 0; i < Mx; ++i) v[i] = (double)mesh[t * Mx + i];
-        spline_line(ax, v, 1, X + (int64_t)t * Mx, 1, scr_c + (int64_t)t * (Mx + My), scr_d + (int64_t)t * (Mx + My));
+    __syncthreads();
+    const int lo = base > 1 ? base : 1, hi = base + SL_N - 1 < n - 2 ? base + SL_N - 1 : n - 2;
+    if (tid < 32) {
+        // the first node of a chunk's overlap has no node before it: its rhs
+        // needs one, so the sweep starts a node later there
+        const int first = lo == base ? lo + 1 : lo, last = hi == base + SL_N - 1 ? hi - 1 : hi;
+        double d = 0.0;
+        if (first <= last) {
+            double vm = v[first - 1 - base][lane], v0 = v[first - base][lane];
+            for (int r = first; r <= last; ++r) {
+                const int k = r - base;
+                const double vp = v[k + 1][lane];
+                const double rhs = 6.0 * ((vp - v0) * ih[k + 1] - (v0 - vm) * ih[k]);
+                d = rhs - w[k] * d;
+                v[k][lane] = d;
+                vm = v0;
+                v0 = vp;
+            }
+            double next = 0.0;
+            const int end = c0 > 1 ? c0 : 1;
+            for (int r = last; r >= end; --r) {
+                const int k = r - base;
+                next = (v[k][lane] - c[k] * next) * ib[k];
+                v[k][lane] = next;
+            }
+        }
     }
-    const int u = t - My;
-    if (u >= 0 && u < Mx) {
-        double* col = colv + (int64_t)u * My;
-        for (int j = 0; j < My; ++j) col[j] = (double)mesh[j * Mx + u];
-        spline_line(ay, col, 1, Y + u, Mx, scr_c + (int64_t)(My + u) * (Mx + My),
-                    scr_d + (int64_t)(My + u) * (Mx + My));
-    }
-}
-
-// XY: along each mesh row of Y; then pack (P, X, Y, XY) as float4
-__global__ void k_spline_pack(const float* mesh, Axis ax, Axis ay, const double* X, double* Y, double* XY,
-                              double* scr_c, double* scr_d, float4* tab)
-{
-    const int Mx = ax.n, My = ay.n;
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= My) return;
-    spline_line(ax, Y + (int64_t)t * Mx, 1, XY + (int64_t)t * Mx, 1, scr_c + (int64_t)t * (Mx + My),
-                scr_d + (int64_t)t * (Mx + My));
-    for (int i = 0; i < Mx; ++i) {
-        int64_t o = (int64_t)t * Mx + i;
-        tab[o] = make_float4(mesh[o], (float)X[o], (float)Y[o], (float)XY[o]);
+    __syncthreads();
+    for (int q = tid; q < SL_CH * 32; q += SL_NT) {
+        const int k = rows ? q % SL_CH : q / 32, l = rows ? q / SL_CH : q % 32;
+        const int node = c0 + k, line = l0 + l;
+        if (node >= n || line >= nline) continue;
+        const double M = node < 1 || node > n - 2 ? 0.0 : v[SL_OV + k][l];
+        const int i = rows ? line * Mx + node : node * Mx + line;
+        if constexpr (FINAL) {
+            maps.tab[blockIdx.y][i] = make_float4(mesh[i], (float)maps.X[blockIdx.y][i], (float)maps.Y[blockIdx.y][i], (float)M);
+        } else {
+            (rows ? maps.X : maps.Y)[blockIdx.y][i] = M;
+        }
     }
 }
 
@@ -1746,24 +1830,33 @@ cudaError_t launch_boxstats(const Image& im, int B, double k, int maxiter, doubl
 cudaError_t launch_mesh_finalize(double* bkg, double* rms, int* valid, double* tmp_b, double* tmp_r, int* tmp_v,
                                  int Mx, int My, int fsize, float* bkg_out, float* rms_out, cudaStream_t st)
 {
-    k_mesh_finalize<<<1, MF_NT, 0, st>>>(bkg, rms, valid, tmp_b, tmp_r, tmp_v, Mx, My, fsize, bkg_out, rms_out);
+    launch_dep(k_mesh_fill, dim3(1), dim3(MF_NT), 0, st, bkg, rms, valid, tmp_b, tmp_r, tmp_v, Mx, My);
+    launch_dep(k_mesh_median, dim3((2 * Mx * My + 255) / 256), dim3(256), 0, st, bkg, rms, Mx, My, fsize, bkg_out, rms_out);
     return cudaGetLastError();
 }
 
-cudaError_t launch_spline_tables(const float* mesh, Axis ax, Axis ay, double* scratch, float4* tab, cudaStream_t st)
+// tables of nmap meshes (mesh[m] -> tab[m]) on the same axes; scratch as for one
+cudaError_t launch_spline_tables(const float* const* mesh, float4* const* tab, int nmap, Axis ax, Axis ay, double* scratch,
+                                 int* nlaunch, cudaStream_t st)
 {
-    const int Mx = ax.n, My = ay.n;
-    const int64_t nn = (int64_t)Mx * My;
-    double* vals = scratch;
-    double* colv = vals + nn;
-    double* X = colv + nn;
-    double* Y = X + nn;
-    double* XY = Y + nn;
-    double* sc = XY + nn;
-    double* sd = sc + (int64_t)(Mx + My) * (Mx + My);
-    const int nt = Mx + My;
-    k_spline_xy<<<(nt + 127) / 128, 128, 0, st>>>(mesh, ax, ay, vals, colv, X, Y, sc, sd);
-    k_spline_pack<<<(My + 127) / 128, 128, 0, st>>>(mesh, ax, ay, X, Y, XY, sc, sd, tab);
+    const int64_t nn = (int64_t)ax.n * ay.n;
+    // X and Y of as many maps at a time as the scratch holds (two at least)
+    const int64_t room = (int64_t)spline_scratch_doubles(ax.n, ay.n) / (2 * nn);
+    const int most = (int)(room < SL_MAPS ? room : SL_MAPS);
+    const int rt = ((ay.n + 31) / 32) * ((ax.n + SL_CH - 1) / SL_CH), ct = ((ax.n + 31) / 32) * ((ay.n + SL_CH - 1) / SL_CH);
+    for (int m0 = 0; m0 < nmap; m0 += most) {
+        const int k = nmap - m0 < most ? nmap - m0 : most;
+        SplineMaps sm = {};
+        for (int m = 0; m < k; ++m) {
+            sm.mesh[m] = mesh[m0 + m];
+            sm.tab[m] = tab[m0 + m];
+            sm.X[m] = scratch + 2 * nn * m;
+            sm.Y[m] = sm.X[m] + nn;
+        }
+        launch_dep(k_spline_lines<false>, dim3(rt + ct, k), dim3(SL_NT), 0, st, sm, ax, ay);
+        launch_dep(k_spline_lines<true>, dim3(rt, k), dim3(SL_NT), 0, st, sm, ax, ay);
+        if (nlaunch) *nlaunch += 2;
+    }
     return cudaGetLastError();
 }
 
