@@ -40,6 +40,47 @@ __device__ __forceinline__ void box_result(double med, double mean, double sd, d
     *rms = sd;
 }
 
+// float-float helpers: |a| >= |b| in df_fast; quotients and roots are a float
+// estimate and one correction from the exact residual (about 46 bits)
+__device__ __forceinline__ DF df_fast(float a, float b)
+{
+    DF r;
+    r.hi = a + b;
+    r.lo = b - (r.hi - a);
+    return r;
+}
+__device__ __forceinline__ DF df_div(DF a, float n)
+{
+    const float q = a.hi / n;
+    const float r = fmaf(-q, n, a.hi) + a.lo;
+    return df_fast(q, r / n);
+}
+__device__ __forceinline__ DF df_sqrt(DF a)
+{
+    if (!(a.hi > 0.f)) return df_zero();
+    const float s = sqrtf(a.hi);
+    return df_fast(s, (fmaf(-s, s, a.hi) + a.lo) / (2.f * s));
+}
+// the smallest float >= a (sign = 1), the largest <= a (sign = -1)
+__device__ __forceinline__ float df_bound(DF a, float sign)
+{
+    return a.lo * sign > 0.f ? nextafterf(a.hi, sign * INFINITY) : a.hi;
+}
+// med + f sd
+__device__ __forceinline__ DF df_step(DF med, float f, DF sd)
+{
+    DF r = med;
+    df_add_prod(r, f, sd.hi);
+    r.lo = fmaf(f, sd.lo, r.lo);
+    return df_fast(r.hi, r.lo);
+}
+// a 64-bit integer to 48 bits
+__device__ __forceinline__ DF df_from(unsigned long long v)
+{
+    const float hi = __ull2float_rz(v);
+    return df_fast(hi, __ull2float_rn(v - (unsigned long long)hi));
+}
+
 // ============================================================ uint16 box ===
 constexpr int U16_NT = 1024;
 constexpr int U16_WORDS = 32768;   // 65,536 16-bit counters
@@ -139,30 +180,34 @@ struct FullHist {
 
 // Iterative k-sigma clip about the median on a histogram (one full warp):
 // the kept set is always the values in an integer range [a, b]; statistics
-// from exact integer sums, median by rank selection.
+// from exact integer sums, median by rank selection.  The passes' bounds come
+// from a float-float sigma (46 bits, and exact where the root and quotient
+// are): a float64 warp instruction holds this GPU's SM for 16 cycles, and the
+// chain of a pass held some 30.  The final statistics are float64.
 template <class Q>
 __device__ __forceinline__ void clip_histogram(Q& q, uint32_t vmin, uint32_t vmax, double k, int maxiter, double* med_o,
                                                double* mean_o, double* sd_o)
 {
-    uint32_t a = vmin, b = vmax;
+    const float kf = (float)k;                // clip_k is a float
+    uint32_t a = vmin, b = vmax, m0, m1;
     HistSums lo = q.prefix(a);
     HistSums hi = q.prefix(b + 1u);
     unsigned long long n = hi.c - lo.c, S1 = hi.s1 - lo.s1, S2 = hi.s2 - lo.s2;
-    double med = 0, mean = 0, sd = 0;
     for (int it = 0;; ++it) {
-        uint32_t m0 = q.select(lo.c + (n - 1) / 2);
-        uint32_t m1 = (n & 1ull) ? m0 : q.select(lo.c + n / 2);
-        med = 0.5 * ((double)m0 + (double)m1);
-        const double in = recip_pos((double)n);
-        mean = (double)S1 * in;
-        // population variance from exact integers: (n S2 - S1^2) / n^2
-        unsigned long long num = n * S2 - S1 * S1;
-        sd = sqrt_pos((double)num) * in;
+        m0 = q.select(lo.c + (n - 1) / 2);
+        m1 = (n & 1ull) ? m0 : q.select(lo.c + n / 2);
         if (it >= maxiter) break;
-        double flo = med - k * sd, fhi = med + k * sd;
-        double ca = ceil(flo), cbv = floor(fhi);
-        uint32_t na = ca <= (double)a ? a : (uint32_t)ca;
-        uint32_t nbv = cbv >= (double)b ? b : (cbv < 0 ? 0u : (uint32_t)cbv);
+        // med -/+ k sigma, with sigma = sqrt(n S2 - S1^2) / n
+        const DF sd = df_div(df_sqrt(df_from(n * S2 - S1 * S1)), (float)n);
+        DF med;
+        med.hi = 0.5f * ((float)m0 + (float)m1);    // exact
+        med.lo = 0.f;
+        const DF fl = df_step(med, -kf, sd), fh = df_step(med, kf, sd);
+        float ca = ceilf(fl.hi), cb = floorf(fh.hi);
+        if (ca == fl.hi && fl.lo > 0.f) ca += 1.f;
+        if (cb == fh.hi && fh.lo < 0.f) cb -= 1.f;
+        uint32_t na = ca <= (float)a ? a : (uint32_t)ca;
+        uint32_t nbv = cb >= (float)b ? b : (cb < 0.f ? 0u : (uint32_t)cb);
         if (nbv < na) { na = a; nbv = a; }   // cannot happen for k > 0 (median lies inside)
         HistSums nlo = q.prefix(na);
         HistSums nhi = q.prefix(nbv + 1u);
@@ -171,9 +216,11 @@ __device__ __forceinline__ void clip_histogram(Q& q, uint32_t vmin, uint32_t vma
         a = na; b = nbv; lo = nlo; hi = nhi;
         n = nn; S1 = nhi.s1 - nlo.s1; S2 = nhi.s2 - nlo.s2;
     }
-    *med_o = med;
-    *mean_o = mean;
-    *sd_o = sd;
+    const double in = recip_pos((double)n);
+    *med_o = 0.5 * ((double)m0 + (double)m1);
+    *mean_o = (double)S1 * in;
+    // population variance from exact integers: (n S2 - S1^2) / n^2
+    *sd_o = sqrt_pos((double)(n * S2 - S1 * S1)) * in;
 }
 
 // rank of quantile q of n good values (features for the learned background)
@@ -394,10 +441,21 @@ __device__ void boxstats_u16_box(const BoxArgs& A, int box, uint32_t* hist)
 // only where they query; a query that falls outside the window (a prefix at
 // a value strictly inside (vmin, w0) or (w0 + 4096, vmax], a rank below or
 // above it) marks the box, which then goes to the full-histogram kernel.
+// Prefixes outside the window are still served when the box has few values
+// there, kept in a list: hot pixels and cosmic rays (0.05 % of the pixels up to
+// full scale) push the first clip bound of nearly every box of a CCD frame
+// past the window, and the full-histogram kernel then took as long as this one
+// (33 us beside 31 on a 4 MP frame at mesh 128, 775 beside 426 at 81 MP and
+// mesh 64; now 4 beside 26, and 4 beside 483).
 // Boxes finished here get bit-identical results: the same integer sums, the
 // same ranks, the same clip loop.
-constexpr int WB_NT = 128;
+//
+// Threads a box by the number of boxes: 128 keep 8 boxes an SM in flight; a
+// frame with fewer boxes than that takes 256 or 512, as it lasts as long as
+// one box (256 boxes of 128 x 128: 31 us with 128 threads, 26 with 512; 512
+// boxes of 256 x 256: 51 us with 128 threads, 56 with 512, 39 with 256).
 constexpr int NWIN = 4096;
+constexpr int NOUT = 1024;              // values outside the window a box may list
 constexpr int WCB = 64;                 // values per coarse bin of the window
 constexpr int NWC = NWIN / WCB;         // 64 coarse bins
 
@@ -406,7 +464,27 @@ struct WinHist {
     const unsigned long long *pc, *ps1, *ps2;   // NWC + 1 prefixes; [0] = the values below the window
     uint32_t w0, vmin, vmax;
     unsigned long long tc, ts1, ts2;            // all good values
+    const uint16_t* out;                        // the nout values outside the window (-1: too many to list)
+    int nout;
     bool failed = false;
+
+    // the listed values in [a, b)
+    __device__ HistSums listed(uint32_t a, uint32_t b)
+    {
+        HistSums r;
+        r.c = r.s1 = r.s2 = 0;
+        for (int i = threadIdx.x & 31; i < nout; i += 32) {
+            const unsigned long long x = out[i];
+            if (x >= a && x < b) { ++r.c; r.s1 += x; r.s2 += x * x; }
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            r.c += __shfl_xor_sync(0xffffffffu, r.c, o);
+            r.s1 += __shfl_xor_sync(0xffffffffu, r.s1, o);
+            r.s2 += __shfl_xor_sync(0xffffffffu, r.s2, o);
+        }
+        return r;
+    }
 
     __device__ HistSums prefix(uint32_t v)
     {
@@ -415,7 +493,13 @@ struct WinHist {
         r.c = r.s1 = r.s2 = 0;
         if (v <= vmin) return r;
         if (v > vmax) { r.c = tc; r.s1 = ts1; r.s2 = ts2; return r; }
-        if (v < w0 || v > w0 + NWIN) { failed = true; return r; }
+        if (v < w0 || v > w0 + NWIN) {
+            if (nout < 0) { failed = true; return r; }
+            if (v < w0) return listed(0u, v);
+            r = listed(w0 + NWIN, v);
+            r.c += pc[NWC]; r.s1 += ps1[NWC]; r.s2 += ps2[NWC];
+            return r;
+        }
         const uint32_t d = v - w0, cb = d / WCB;
         r.c = pc[cb]; r.s1 = ps1[cb]; r.s2 = ps2[cb];
         if (cb >= NWC) return r;
@@ -470,8 +554,9 @@ struct WinHist {
     }
 };
 
-__global__ void __launch_bounds__(WB_NT, 8) k_boxstats_win(const BoxArgs* __restrict__ batch,
-                                                        const __grid_constant__ BoxArgs one)
+template <int WB_NT>
+__global__ void __launch_bounds__(WB_NT, 1024 / WB_NT) k_boxstats_win(const BoxArgs* __restrict__ batch,
+                                                                      const __grid_constant__ BoxArgs one)
 {
     pdl_wait();
     pdl_release();
@@ -489,6 +574,8 @@ __global__ void __launch_bounds__(WB_NT, 8) k_boxstats_win(const BoxArgs* __rest
     __shared__ unsigned long long red64[6][WB_NT / 32];
     __shared__ uint32_t red_min[WB_NT / 32], red_max[WB_NT / 32], red_n[WB_NT / 32];
     __shared__ uint32_t s_w0;
+    __shared__ uint16_t out[NOUT];
+    __shared__ int nout;
 
     const int bi = box % Mx, bj = box / Mx;
     const int x0 = bi * B, x1 = min(x0 + B, W);
@@ -499,32 +586,56 @@ __global__ void __launch_bounds__(WB_NT, 8) k_boxstats_win(const BoxArgs* __rest
     const bool vec = ((((uintptr_t)img) & 15) == 0) && ((pitch & 7) == 0) && ((x0 & 7) == 0) && ((bw & 7) == 0) &&
                      !mask;
 
+    // f(value) for the good pixels of `rows` rows of the box, `step` apart
+    // (rows unaligned, or a mask): neighbouring threads take neighbouring
+    // pixels, 8 loads of each array in flight
+    auto each_pixel = [&](int rows, int step, auto f) {
+        const int dr = WB_NT / bw, dc = WB_NT - dr * bw;
+        int ry = tid / bw, rx = tid - ry * bw;
+        while (ry < rows) {
+            constexpr int U = 8;
+            uint16_t v[U];
+            uint8_t m[U];
+            int n = 0;
+#pragma unroll
+            for (int k = 0; k < U; ++k) {
+                if (ry < rows) {
+                    const int64_t y = y0 + ry * step;
+                    v[k] = __ldg(img + y * pitch + x0 + rx);
+                    m[k] = mask ? __ldg(mask + y * W + x0 + rx) : 0;
+                    ++n;
+                }
+                rx += dc;
+                ry += dr;
+                if (rx >= bw) { rx -= bw; ++ry; }
+            }
+#pragma unroll
+            for (int k = 0; k < U; ++k)
+                if (k < n && !m[k]) f(v[k]);
+        }
+    };
+
     for (int w = tid; w < NWIN; w += WB_NT) win[w] = 0u;
     for (int i = tid; i < 256; i += WB_NT) samp[i] = 0u;
+    if (tid == 0) nout = 0;
     __syncthreads();
 
     // ---- sample (every 16th row): median coarse value -> window
     {
         const int srow = (bh + 15) >> 4;
-        for (int c = tid; c < srow * cpr; c += WB_NT) {
-            const int ry = (c / cpr) * 16, rc = c - (c / cpr) * cpr;
-            const int y = y0 + ry, xs = x0 + rc * 8;
-            const uint16_t* row = img + (int64_t)y * pitch;
-            if (vec) {
-                const uint4 q = __ldg(reinterpret_cast<const uint4*>(row + xs));
+        if (vec) {
+            for (int c = tid; c < srow * cpr; c += WB_NT) {
+                const int ry = (c / cpr) * 16, rc = c - (c / cpr) * cpr;
+                const uint4 q = __ldg(reinterpret_cast<const uint4*>(img + (int64_t)(y0 + ry) * pitch + x0 + rc * 8));
                 const uint32_t w4[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
                     atomicAdd(&samp[(w4[e] & 0xffffu) >> 8], 1u);
                     atomicAdd(&samp[w4[e] >> 24], 1u);
                 }
-            } else {
-                const int nv = min(8, x1 - xs);
-                for (int e = 0; e < nv; ++e) {
-                    if (mask && mask[(int64_t)y * W + xs + e]) continue;
-                    atomicAdd(&samp[__ldg(row + xs + e) >> 8], 1u);
-                }
             }
+        } else {
+            each_pixel(srow, 16, [&](uint32_t u) { atomicAdd(&samp[u >> 8], 1u); });
         }
     }
     __syncthreads();
@@ -569,13 +680,16 @@ __global__ void __launch_bounds__(WB_NT, 8) k_boxstats_win(const BoxArgs* __rest
         const uint32_t d = u - w0;
         if (d < (uint32_t)NWIN) {
             atomicAdd(&win[d], 1u);
-        } else if (u < w0) {
+            return;
+        }
+        const int i = atomicAdd(&nout, 1);
+        if (i < NOUT) out[i] = (uint16_t)u;
+        if (u < w0) {
             ++lc; ls1 += u; ls2 += (unsigned long long)u * u;
         } else {
             ++hc; hs1 += u; hs2 += (unsigned long long)u * u;
         }
     };
-    const int nchunks = cpr * bh;
     if (vec) {
         // 16-byte chunks (8 values); a thread's (row, chunk) advance by the
         // fixed step of one pass of the CTA, without a division per chunk.
@@ -627,16 +741,7 @@ __global__ void __launch_bounds__(WB_NT, 8) k_boxstats_win(const BoxArgs* __rest
                 vmax = max(vmax, w0 + (uint32_t)w);
             }
     } else {
-        for (int c = tid; c < nchunks; c += WB_NT) {
-            const int ry = c / cpr, rc = c - ry * cpr;
-            const int y = y0 + ry, xs = x0 + rc * 8;
-            const uint16_t* row = img + (int64_t)y * pitch;
-            const int nv = min(8, x1 - xs);
-            for (int e = 0; e < nv; ++e) {
-                if (mask && mask[(int64_t)y * W + xs + e]) continue;
-                count(__ldg(row + xs + e));
-            }
-        }
+        each_pixel(bh, 1, count);
     }
     unsigned long long agg[6] = {lc, ls1, ls2, hc, hs1, hs2};
 #pragma unroll
@@ -731,6 +836,7 @@ __global__ void __launch_bounds__(WB_NT, 8) k_boxstats_win(const BoxArgs* __rest
     WinHist wq;
     wq.win = win; wq.pc = pc; wq.ps1 = ps1; wq.ps2 = ps2;
     wq.w0 = w0; wq.vmin = vmin; wq.vmax = vmax;
+    wq.out = out; wq.nout = nout <= NOUT ? nout : -1;
     wq.tc = pc[NWC] + agg[3]; wq.ts1 = ps1[NWC] + agg[4]; wq.ts2 = ps2[NWC] + agg[5];
     double med, mean, sd;
     clip_histogram(wq, vmin, vmax, A.k, A.maxiter, &med, &mean, &sd);
@@ -842,40 +948,6 @@ struct F32Box {
     uint32_t flag[SEL_BPT * NT / 32];     // a bit per bin: holds a quantile
 };
 
-// float-float helpers: |a| >= |b| in df_fast; quotients and roots are a float
-// estimate and one correction from the exact residual (about 46 bits)
-__device__ __forceinline__ DF df_fast(float a, float b)
-{
-    DF r;
-    r.hi = a + b;
-    r.lo = b - (r.hi - a);
-    return r;
-}
-__device__ __forceinline__ DF df_div(DF a, float n)
-{
-    const float q = a.hi / n;
-    const float r = fmaf(-q, n, a.hi) + a.lo;
-    return df_fast(q, r / n);
-}
-__device__ __forceinline__ DF df_sqrt(DF a)
-{
-    if (!(a.hi > 0.f)) return df_zero();
-    const float s = sqrtf(a.hi);
-    return df_fast(s, (fmaf(-s, s, a.hi) + a.lo) / (2.f * s));
-}
-// the smallest float >= a (sign = 1), the largest <= a (sign = -1)
-__device__ __forceinline__ float df_bound(DF a, float sign)
-{
-    return a.lo * sign > 0.f ? nextafterf(a.hi, sign * INFINITY) : a.hi;
-}
-// med + f sd
-__device__ __forceinline__ DF df_step(DF med, float f, DF sd)
-{
-    DF r = med;
-    df_add_prod(r, f, sd.hi);
-    r.lo = fmaf(f, sd.lo, r.lo);
-    return df_fast(r.hi, r.lo);
-}
 // sum over the first NW lanes (a power of two), in lane 0 .. NW - 1
 template <int NW>
 __device__ __forceinline__ DF df_sum_lanes(DF v)
@@ -1797,7 +1869,10 @@ cudaError_t launch_boxstats_any(const BoxArgs& one, const BoxArgs* batch, int nf
     if (!is_f32 && one.fb_list) {
         // windowed histograms, then the full histogram for the boxes they
         // could not finish (a persistent grid over the fallback lists)
-        launch_dep(k_boxstats_win, grid, dim3(WB_NT), 0, st, batch, one);
+        const int64_t boxes = (int64_t)maxbox * nframes, area = (int64_t)one.B * one.B;
+        if (boxes >= 8 * 152 || area < 256 * 32) launch_dep(k_boxstats_win<128>, grid, dim3(128), 0, st, batch, one);
+        else if (boxes >= 2 * 152 || area < 512 * 32) launch_dep(k_boxstats_win<256>, grid, dim3(256), 0, st, batch, one);
+        else launch_dep(k_boxstats_win<512>, grid, dim3(512), 0, st, batch, one);
         const size_t smem = U16_WORDS * sizeof(uint32_t);
         cudaFuncSetAttribute(k_boxstats_u16, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         launch_dep(k_boxstats_u16, dim3(maxbox < 152 ? maxbox : 152, nframes), dim3(U16_NT), smem, st, batch, one);
