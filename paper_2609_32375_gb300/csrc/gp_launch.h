@@ -89,8 +89,9 @@ cudaError_t launch_deblend(const Image& im, const SplineTab& sb, const SplineTab
 // are given; scratch of the isolation grid from iso_grid()
 struct RoptWork {
     int *count, *start, *fill, *items;
-    double2* xy;          // [rows] (log10 nu, log10 r) of the calibrators
+    double* parts;        // the fit's sums by CTA: 7 doubles each, at most a CTA per 64 rows, at most ROPT_PARTS
 };
+constexpr int ROPT_PARTS = 152 * 8, ROPT_PART_DOUBLES = 7;
 void iso_grid(int W, int H, float d_iso, double* cs, int* ncx, int* ncy);
 cudaError_t launch_ropt(const Image& im, const SplineTab& sb, const SplineTab& sr, const float* taps, int kw, int kh,
                         const gp_catalog& cat, const double* flux, const double* ferr, const uint32_t* gflags,

@@ -879,57 +879,6 @@ __global__ void __launch_bounds__(WB_NT, 1024 / WB_NT) k_boxstats_win(const BoxA
 // and its long latency sits in the chain of every pass.
 constexpr int F32_LIST = 64;      // values among which the median is ranked
 
-__device__ __forceinline__ unsigned long long f2pack(float a, float b)
-{
-    return (unsigned long long)__float_as_uint(a) | ((unsigned long long)__float_as_uint(b) << 32);
-}
-__device__ __forceinline__ float f2lo(unsigned long long a) { return __uint_as_float((uint32_t)a); }
-__device__ __forceinline__ float f2hi(unsigned long long a) { return __uint_as_float((uint32_t)(a >> 32)); }
-__device__ __forceinline__ unsigned long long f2add(unsigned long long a, unsigned long long b)
-{
-    unsigned long long d;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-__device__ __forceinline__ unsigned long long f2sub(unsigned long long a, unsigned long long b)
-{
-    unsigned long long d;
-    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-__device__ __forceinline__ unsigned long long f2mul(unsigned long long a, unsigned long long b)
-{
-    unsigned long long d;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-__device__ __forceinline__ unsigned long long f2fma(unsigned long long a, unsigned long long b, unsigned long long c)
-{
-    unsigned long long d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
-
-// two float-float accumulators side by side (df_add for each)
-struct DF2 {
-    unsigned long long hi, lo;
-};
-__device__ __forceinline__ void df2_add(DF2& s, unsigned long long v)
-{
-    const unsigned long long t = f2add(s.hi, v);
-    const unsigned long long bp = f2sub(t, s.hi);
-    const unsigned long long e = f2add(f2sub(s.hi, f2sub(t, bp)), f2sub(v, bp));
-    s.hi = t;
-    s.lo = f2add(s.lo, e);
-}
-__device__ __forceinline__ DF df2_sum(const DF2& s)
-{
-    DF a, b;
-    a.hi = f2lo(s.hi); a.lo = f2lo(s.lo);
-    b.hi = f2hi(s.hi); b.lo = f2hi(s.lo);
-    return df_merge(a, b);
-}
-
 template <int NT>
 struct F32Box {
     __align__(16) uint32_t pre[SEL_BPT * NT + 4];     // values in the bins before; [NB] the total
