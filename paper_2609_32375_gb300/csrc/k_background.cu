@@ -1503,21 +1503,25 @@ __global__ void k_bkg_maps(SplineTab sb, SplineTab sr, int W, int H, float* bmap
 }
 
 // ====================================================== fused mesh kernel ===
-// One CTA does the whole mesh stage in shared memory when the mesh has at
-// most MESH_SMEM_NODES nodes: invalid-box fill, median filter, and the
-// spline tables of both maps.  The tridiagonal matrix of the natural spline
+// One CTA a map does the whole mesh stage in shared memory when the mesh has
+// at most MESH_SMEM_NODES nodes: invalid-box fill, median filter, and the
+// spline tables.  The tridiagonal matrix of the natural spline
 // depends only on the node positions, so each axis is factorised once
 // (multipliers and reciprocal pivots) and every line is then solved with
 // FMAs only.  FP32 throughout: the tables are stored in FP32 anyway, and the
 // diagonally dominant spline system loses nothing that matters at 1e-5.
+// Bound by latency, a line's recurrences above all: the lines' values are
+// loaded SL_AHEAD nodes ahead of them.  A 2048 x 2048 frame's 32 x 32 mesh
+// takes 7.5 us and a 64 x 64 one 17.6 (13 and 34 with both maps in one CTA, a
+// load before each step and every pivot divided out).
 constexpr int MESH_SMEM_NODES = 4096;
 constexpr int MA_NT = 1024;
 
-// byte offset of the LU scratch in k_mesh_all's shared memory: six float
+// byte offset of the LU scratch in k_mesh_all's shared memory: three float
 // arrays and two int arrays of n entries, rounded up to 16 bytes
 __host__ __device__ __forceinline__ size_t mesh_lu_offset(int n)
 {
-    const size_t end = (size_t)n * (6 * sizeof(float) + 2 * sizeof(int));
+    const size_t end = (size_t)n * (3 * sizeof(float) + 2 * sizeof(int));
     return (end + 15) & ~(size_t)15;
 }
 
@@ -1533,145 +1537,170 @@ __device__ __forceinline__ float node_pos(const Axis& a, int i)
     return (i == a.n - 1) ? a.tl : a.t0 + (float)i * a.B;
 }
 
-__device__ void factor_axis(const Axis& a, AxisLU L)
+// a warp; the pivots' recurrence on its first lane.  With equal intervals it
+// soon repeats its values, and a step whose operands are those of the step
+// before has its results.
+__device__ void factor_axis(const Axis& a, AxisLU L, int lane)
 {
     const int n = a.n;
-    for (int i = 0; i + 1 < n; ++i) L.ih[i] = 1.f / (node_pos(a, i + 1) - node_pos(a, i));
-    float bprev = 0.f, cprev = 0.f;
+    for (int i = lane; i + 1 < n; i += 32) L.ih[i] = 1.f / (node_pos(a, i + 1) - node_pos(a, i));
+    if (lane) return;
+    float bprev = 0.f, cprev = 0.f, h0p = 0.f, h1p = 0.f, bpp = 0.f, w = 0.f, ib = 0.f, b = 0.f;
     for (int r = 1; r <= n - 2; ++r) {
         const float h0 = node_pos(a, r) - node_pos(a, r - 1), h1 = node_pos(a, r + 1) - node_pos(a, r);
-        float b = 2.f * (h0 + h1);
-        float w = 0.f;
-        if (r > 1) {
-            w = h0 / bprev;
-            b -= w * cprev;
+        if (!(r > 2 && h0 == h0p && h1 == h1p && bprev == bpp && cprev == h0)) {
+            b = 2.f * (h0 + h1);
+            w = 0.f;
+            if (r > 1) {
+                w = h0 / bprev;
+                b -= w * cprev;
+            }
+            ib = 1.f / b;
         }
         L.w[r] = w;
-        L.ib[r] = 1.f / b;
+        L.ib[r] = ib;
         L.c[r] = h1;
+        h0p = h0;
+        h1p = h1;
+        bpp = bprev;
         bprev = b;
         cprev = h1;
     }
 }
 
 // second derivatives of one line (values v, stride vs) into M (stride ms)
+constexpr int SL_AHEAD = 8;
 __device__ void solve_line(const AxisLU& L, int n, const float* v, int vs, float* M, int ms)
 {
     M[0] = 0.f;
     if (n >= 2) M[(n - 1) * ms] = 0.f;
     if (n < 3) return;
-    float dprev = 0.f;
-    for (int r = 1; r <= n - 2; ++r) {
-        float d = 6.f * ((v[(r + 1) * vs] - v[r * vs]) * L.ih[r] - (v[r * vs] - v[(r - 1) * vs]) * L.ih[r - 1]);
-        d = fmaf(-L.w[r], dprev, d);
-        M[r * ms] = d;        // forward-eliminated right-hand side
-        dprev = d;
+    float dprev = 0.f, vr = v[vs], pr = (vr - v[0]) * L.ih[0];      // slope before node r
+    for (int r0 = 1; r0 <= n - 2; r0 += SL_AHEAD) {
+        float vn[SL_AHEAD], ih[SL_AHEAD], w[SL_AHEAD], d[SL_AHEAD];
+#pragma unroll
+        for (int j = 0; j < SL_AHEAD; ++j) {
+            const int r = min(r0 + j, n - 2);
+            vn[j] = v[(r + 1) * vs];
+            ih[j] = L.ih[r];
+            w[j] = L.w[r];
+        }
+#pragma unroll
+        for (int j = 0; j < SL_AHEAD; ++j) {
+            const float dv = vn[j] - vr;
+            d[j] = 6.f * fmaf(dv, ih[j], -pr);
+            pr = __fmul_rn(dv, ih[j]);
+            vr = vn[j];
+        }
+#pragma unroll
+        for (int j = 0; j < SL_AHEAD; ++j)
+            if (r0 + j <= n - 2) {
+                dprev = fmaf(-w[j], dprev, d[j]);
+                M[(r0 + j) * ms] = dprev;        // forward-eliminated right-hand side
+            }
     }
     float next = 0.f;
-    for (int r = n - 2; r >= 1; --r) {
-        const float val = fmaf(-L.c[r], next, M[r * ms]) * L.ib[r];
-        M[r * ms] = val;
-        next = val;
+    for (int r0 = n - 2; r0 >= 1; r0 -= SL_AHEAD) {
+        float c[SL_AHEAD], ib[SL_AHEAD], m[SL_AHEAD];
+#pragma unroll
+        for (int j = 0; j < SL_AHEAD; ++j) {
+            const int r = max(r0 - j, 1);
+            c[j] = L.c[r];
+            ib[j] = L.ib[r];
+            m[j] = M[r * ms];
+        }
+#pragma unroll
+        for (int j = 0; j < SL_AHEAD; ++j)
+            if (r0 - j >= 1) {
+                next = fmaf(-c[j], next, m[j]) * ib[j];
+                M[(r0 - j) * ms] = next;
+            }
     }
 }
 
 // mode 0: raw box statistics -> fill, filter, write meshes, tables
 // mode 1: tables only, from the float meshes given in bkg_out / rms_out
+// blockIdx.x = the map: background, noise
 __global__ void __launch_bounds__(MA_NT) k_mesh_all(const MeshArgs* __restrict__ batch,
                                                     const __grid_constant__ MeshArgs one)
 {
     pdl_wait();
     pdl_release();
     const MeshArgs& MA = frame_args(batch, one);
-    const double* __restrict__ bkg_raw = MA.bkg_raw;
-    const double* __restrict__ rms_raw = MA.rms_raw;
+    const double* __restrict__ raw = blockIdx.x ? MA.rms_raw : MA.bkg_raw;
     const int* __restrict__ valid_raw = MA.valid;
     const Axis ax = MA.ax, ay = MA.ay;
     const int fsize = MA.fsize, mode = MA.mode;
-    float* bkg_out = MA.bkg_mesh;
-    float* rms_out = MA.rms_mesh;
-    float4* tab_b = MA.tab_b;
-    float4* tab_r = MA.tab_r;
+    float* out = blockIdx.x ? MA.rms_mesh : MA.bkg_mesh;
+    float4* tab = blockIdx.x ? MA.tab_r : MA.tab_b;
     extern __shared__ __align__(16) float sh[];
     unsigned char* sh_bytes = reinterpret_cast<unsigned char*>(sh);
     // shared-memory rows are Ms = Mx | 1 wide (odd), so the row-direction
     // solves, one row per lane, hit 32 different banks
     const int Mx = ax.n, My = ay.n, n = Mx * My, tid = threadIdx.x;
     const int Ms = Mx | 1, ns = Ms * My;
-    float* A0 = sh;
-    float* A1 = A0 + ns;
-    float* A2 = A1 + ns;
-    float* A3 = A2 + ns;
-    float* A4 = A3 + ns;
-    float* A5 = A4 + ns;
-    int* V0 = reinterpret_cast<int*>(A5 + ns);
+    float* A = sh;             // raw values; X
+    float* T = A + ns;         // fill scratch; Y
+    float* P = T + ns;         // filtered values; XY
+    int* V0 = reinterpret_cast<int*>(P + ns);
     int* V1 = V0 + ns;
     const int nl = Mx > My ? Mx : My;
     // the LU scratch starts at the first 16-byte boundary after V1
     float* lu = reinterpret_cast<float*>(sh_bytes + mesh_lu_offset(ns));
     AxisLU Lx{lu, lu + nl, lu + 2 * nl, lu + 3 * nl};
     AxisLU Ly{lu + 4 * nl, lu + 5 * nl, lu + 6 * nl, lu + 7 * nl};
-    __shared__ int missing, any;
+    // two warps factor the spline systems (first needed by the solves)
+    if (tid >= MA_NT - 32) factor_axis(ax, Lx, tid & 31);
+    else if (tid >= MA_NT - 64) factor_axis(ay, Ly, tid & 31);
 
     if (mode == 0) {
-        if (tid == 0) any = 0;
-        __syncthreads();
+        bool good = false, gap = false;
         for (int b = tid; b < n; b += MA_NT) {
-            const int sb_ = (b / Mx) * Ms + b % Mx;
-            A0[sb_] = (float)bkg_raw[b]; A1[sb_] = (float)rms_raw[b]; V0[sb_] = valid_raw[b];
-            if (V0[sb_]) any = 1;
+            const int sb_ = (b / Mx) * Ms + b % Mx, v = valid_raw[b];
+            A[sb_] = (float)raw[b];
+            V0[sb_] = v;
+            good |= v != 0;
+            gap |= v == 0;
         }
-        __syncthreads();
+        const bool any = __syncthreads_or(good);
         if (!any) {
-            for (int b = tid; b < n; b += MA_NT) {
-                const int sb_ = (b / Mx) * Ms + b % Mx;
-                A0[sb_] = 0.f; A1[sb_] = 0.f; V0[sb_] = 1;
-            }
+            for (int i = tid; i < ns; i += MA_NT) A[i] = 0.f;
             __syncthreads();
         }
+        bool more = __syncthreads_or(gap) && any;
         // fill invalid boxes from valid 8-neighbours, sweep after sweep
-        for (int sweep = 0; sweep < Mx + My + 2; ++sweep) {
-            if (tid == 0) missing = 0;
-            __syncthreads();
+        for (int sweep = 0; more && sweep < Mx + My + 2; ++sweep) {
+            bool missing = false;
             for (int b = tid; b < n; b += MA_NT) {
                 const int i = b % Mx, j = b / Mx, sb_ = j * Ms + i;
-                A2[sb_] = A0[sb_]; A3[sb_] = A1[sb_]; V1[sb_] = V0[sb_];
+                T[sb_] = A[sb_]; V1[sb_] = V0[sb_];
                 if (V0[sb_]) continue;
                 int c = 0;
-                float sb = 0.f, sr = 0.f;
+                float sum = 0.f;
                 for (int dj = -1; dj <= 1; ++dj)
                     for (int di = -1; di <= 1; ++di) {
                         const int ii = i + di, jj = j + dj;
                         if ((di || dj) && ii >= 0 && ii < Mx && jj >= 0 && jj < My && V0[jj * Ms + ii]) {
-                            sb += A0[jj * Ms + ii];
-                            sr += A1[jj * Ms + ii];
+                            sum += A[jj * Ms + ii];
                             ++c;
                         }
                     }
-                if (c) { A2[sb_] = sb / c; A3[sb_] = sr / c; V1[sb_] = 1; }
-                else missing = 1;
+                if (c) { T[sb_] = sum / c; V1[sb_] = 1; }
+                else missing = true;
             }
-            __syncthreads();
-            const bool more = missing;
+            more = __syncthreads_or(missing);
             for (int b = tid; b < n; b += MA_NT) {
                 const int sb_ = (b / Mx) * Ms + b % Mx;
-                A0[sb_] = A2[sb_]; A1[sb_] = A3[sb_]; V0[sb_] = V1[sb_];
+                A[sb_] = T[sb_]; V0[sb_] = V1[sb_];
             }
             __syncthreads();
-            if (!more) break;
         }
-        // median filter (window clipped at the mesh edge) -> float meshes;
-        // meanwhile two threads factor the spline systems (first needed by
-        // the solves further down)
-        if (tid == MA_NT - 32) factor_axis(ax, Lx);
-        if (tid == MA_NT - 64) factor_axis(ay, Ly);
+        // median filter (window clipped at the mesh edge) -> float mesh
         const int h = fsize / 2;
-        for (int t = tid; t < 2 * n && fsize == 3; t += MA_NT) {
+        for (int b = tid; b < n && fsize == 3; b += MA_NT) {
             // 3 x 3: the window in registers (absent cells +inf), sorted by
             // odd-even transposition; the same order statistics as below
-            const int map = t / n, b = t - map * n;
             const int i = b % Mx, j = b / Mx;
-            const float* src = map ? A1 : A0;
             float w[9];
             int c = 0;
 #pragma unroll
@@ -1680,7 +1709,7 @@ __global__ void __launch_bounds__(MA_NT) k_mesh_all(const MeshArgs* __restrict__
                 for (int di = -1; di <= 1; ++di) {
                     const int ii = i + di, jj = j + dj;
                     const bool in = ii >= 0 && ii < Mx && jj >= 0 && jj < My;
-                    w[(dj + 1) * 3 + di + 1] = in ? src[jj * Ms + ii] : INFINITY;
+                    w[(dj + 1) * 3 + di + 1] = in ? A[jj * Ms + ii] : INFINITY;
                     c += in ? 1 : 0;
                 }
 #pragma unroll
@@ -1697,64 +1726,41 @@ __global__ void __launch_bounds__(MA_NT) k_mesh_all(const MeshArgs* __restrict__
                 if (q == (c - 1) / 2) m0 = w[q];
                 if (q == c / 2) m1 = w[q];
             }
-            (map ? rms_out : bkg_out)[b] = (c & 1) ? m1 : 0.5f * (m0 + m1);
+            P[j * Ms + i] = out[b] = (c & 1) ? m1 : 0.5f * (m0 + m1);
         }
-        for (int t = tid; t < 2 * n && fsize != 3; t += MA_NT) {
-            const int map = t / n, b = t - map * n;
+        for (int b = tid; b < n && fsize != 3; b += MA_NT) {
             const int i = b % Mx, j = b / Mx;
-            const float* src = map ? A1 : A0;
             float win[49];
             int c = 0;
             for (int jj = j - h; jj <= j + h; ++jj)
                 for (int ii = i - h; ii <= i + h; ++ii)
                     if (ii >= 0 && ii < Mx && jj >= 0 && jj < My) {
-                        const float v = src[jj * Ms + ii];
+                        const float v = A[jj * Ms + ii];
                         int p = c++;
                         while (p > 0 && win[p - 1] > v) { win[p] = win[p - 1]; --p; }
                         win[p] = v;
                     }
-            const float med = (c & 1) ? win[c / 2] : 0.5f * (win[c / 2 - 1] + win[c / 2]);
-            (map ? rms_out : bkg_out)[b] = med;
+            P[j * Ms + i] = out[b] = (c & 1) ? win[c / 2] : 0.5f * (win[c / 2 - 1] + win[c / 2]);
         }
+    } else {
+        for (int b = tid; b < n; b += MA_NT) P[(b / Mx) * Ms + b % Mx] = out[b];
     }
     __syncthreads();
-    // spline tables of both maps, from the float meshes: X (rows) and Y
-    // (columns) for both maps at once, then XY (rows of Y)
-    if (mode != 0) {
-        if (tid == 0) factor_axis(ax, Lx);
-        if (tid == 32) factor_axis(ay, Ly);
+    // spline table: X (rows) and Y (columns) at once, then XY (rows of Y)
+    for (int q = tid; q < My + Mx; q += MA_NT) {
+        if (q < My) solve_line(Lx, Mx, P + q * Ms, 1, A + q * Ms, 1);
+        else solve_line(Ly, My, P + (q - My), Ms, T + (q - My), Ms);
     }
+    __syncthreads();
+    // the values go out before XY overwrites them
     for (int b = tid; b < n; b += MA_NT) {
         const int sb_ = (b / Mx) * Ms + b % Mx;
-        A4[sb_] = bkg_out[b]; A5[sb_] = rms_out[b];
+        tab[b] = make_float4(P[sb_], A[sb_], T[sb_], 0.f);
     }
     __syncthreads();
-    for (int t = tid; t < 2 * (My + Mx); t += MA_NT) {
-        const int map = t / (My + Mx), q = t - map * (My + Mx);
-        const float* P = map ? A5 : A4;
-        float* X = map ? A1 : A0;
-        float* Y = map ? A3 : A2;
-        if (q < My) solve_line(Lx, Mx, P + q * Ms, 1, X + q * Ms, 1);
-        else solve_line(Ly, My, P + (q - My), Ms, Y + (q - My), Ms);
-    }
+    for (int q = tid; q < My; q += MA_NT) solve_line(Lx, Mx, T + q * Ms, 1, P + q * Ms, 1);
     __syncthreads();
-    // XY overwrites P (no longer needed once X and Y are known)
-    for (int b = tid; b < n; b += MA_NT) {
-        const int sb_ = (b / Mx) * Ms + b % Mx;
-        tab_b[b] = make_float4(A4[sb_], A0[sb_], A2[sb_], 0.f);
-        tab_r[b] = make_float4(A5[sb_], A1[sb_], A3[sb_], 0.f);
-    }
-    __syncthreads();
-    for (int t = tid; t < 2 * My; t += MA_NT) {
-        const int map = t / My, q = t - map * My;
-        solve_line(Lx, Mx, (map ? A3 : A2) + q * Ms, 1, (map ? A5 : A4) + q * Ms, 1);
-    }
-    __syncthreads();
-    for (int b = tid; b < n; b += MA_NT) {
-        const int sb_ = (b / Mx) * Ms + b % Mx;
-        tab_b[b].w = A4[sb_];
-        tab_r[b].w = A5[sb_];
-    }
+    for (int b = tid; b < n; b += MA_NT) tab[b].w = P[(b / Mx) * Ms + b % Mx];
 }
 
 size_t mesh_all_smem(int Mx, int My)
@@ -1783,7 +1789,7 @@ MeshArgs mesh_args(const double* bkg_raw, const double* rms_raw, const int* vali
 cudaError_t launch_mesh_all_any(const MeshArgs& one, const MeshArgs* batch, int nframes, size_t smem, cudaStream_t st)
 {
     cudaFuncSetAttribute(k_mesh_all, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    launch_dep(k_mesh_all, dim3(1, nframes), dim3(MA_NT), smem, st, batch, one);
+    launch_dep(k_mesh_all, dim3(2, nframes), dim3(MA_NT), smem, st, batch, one);
     return cudaGetLastError();
 }
 
