@@ -12,8 +12,8 @@
 //                  histograms of the range, sums in compensated FP32.
 //  k_mesh_all      boxes with < 50 % good pixels filled from valid neighbours,
 //                  both meshes median-filtered, second-derivative tables of the
-//                  tensor-product natural spline through the box centres: one
-//                  CTA, for meshes that fit its shared memory.
+//                  tensor-product natural spline through the box centres: a
+//                  CTA a map, for meshes that fit its shared memory.
 //  k_mesh_fill, k_mesh_median, k_spline_lines
 //                  the same for larger meshes (FP64 tridiagonal solves).
 //  k_bkg_maps      optional full-resolution B(p), sigma(p) output.

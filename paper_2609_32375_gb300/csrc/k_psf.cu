@@ -10,13 +10,21 @@
 // so the labelling, merge and moments that follow are the plain path's.
 //
 // A CTA takes one 128-column strip and one 32-row tile band.  m over the band
-// and a halo of KS/2 is formed in shared memory (B from per-row and
-// per-column spline coefficients); a thread takes one column and 8 rows and
-// correlates them with two kernels at a time: per tap column it loads the
-// 8 + KS - 1 values of its column once and applies the KS tap pairs of that
-// column to its 8 rows with paired FMAs (each half rounds as one fmaf, so the
-// results do not depend on the pairing).  The taps (zero-padded to KS x KS,
-// centred) are kernel parameters.
+// and a halo of KS/2 is formed in shared memory (four rows of a column at a
+// time, which share the column's terms of the background spline); a thread
+// takes one column and 16 rows and correlates them with two kernels at a
+// time: per tap column it keeps the KS tap pairs in registers and walks the
+// 16 + KS - 1 values of its column once, adding each to the rows that it
+// reaches with paired FMAs (each half rounds as one fmaf, and each row meets its taps
+// in order, so the results depend neither on the pairing nor on the walk).
+// The taps (zero-padded to KS x KS, centred) are kernel parameters.
+//
+// Bound by the FMA pipe, two cycles a paired FMA: 13 x 13 taps, six kernels
+// and 4096 x 4096 pixels are 266 M of them, 455 us.  It takes 630 us, and
+// took 888 with 8 rows a thread (a third of its instructions were FMAs): the
+// window's values copied into pairs half as often, and the splines' row
+// terms from shared memory instead of divided out by every thread, are what
+// went.
 #include <math.h>
 #include <string.h>
 
@@ -27,8 +35,9 @@ namespace gp {
 
 constexpr int PS_ROWS = TY;                 // rows of a CTA: one tile band
 constexpr int PS_COLS = ST_STRIP;           // columns: one mask strip (two tiles)
-constexpr int PS_RPT = 8;                   // rows per thread
-constexpr int PS_NT = PS_COLS * (PS_ROWS / PS_RPT);   // 512 threads
+constexpr int PS_RPT = 16;                  // rows per thread
+constexpr int PS_NT = PS_COLS * (PS_ROWS / PS_RPT);   // 256 threads
+constexpr int PS_FILL = 4;                  // rows of a column filled together
 
 // two FMAs with one rounding each, in one instruction (Blackwell's paired
 // FP32 path): the lanes of a pair are independent, so the results are those
@@ -57,19 +66,17 @@ struct PsfArgs {
     int* tl_list;
     int* tl_count;
     Tiles T;
-    float2 taps[PS_NPAIR][KMAX];             // kernels 2p and 2p + 1 of P0, then the modes, each KS x KS
+    float2 taps[PS_NPAIR][KMAX];             // kernels 2p and 2p + 1 of P0, then the modes: KS columns of KS taps
 };
 
 template <bool F32, int KS>
-__global__ void __launch_bounds__(PS_NT) k_psf(const __grid_constant__ PsfArgs A)
+__global__ void __launch_bounds__(PS_NT, 3) k_psf(const __grid_constant__ PsfArgs A)
 {
     constexpr int H = KS / 2, SR = PS_ROWS + KS - 1, SC = PS_COLS + KS - 1;
-    constexpr int UNROLL_U = KS <= 5 ? KS : 1;     // tap columns unrolled for small kernels only (registers)
     __shared__ float ms[SR][SC];
     __shared__ float4 rowc[SR];            // b, c0, c1 of the background y-spline of each staged row
     __shared__ int2 rowj[SR];
-    __shared__ float4 colc[SC];            // and of the x-spline of each staged column
-    __shared__ int2 colj[SC];
+    __shared__ float4 modec[GP_PSF_MAX_MODES][PS_ROWS];   // b, c0, c1, i of the modes' y-splines
     __shared__ uint8_t bads[PS_ROWS][PS_COLS];
     __shared__ uint32_t mbits[PS_ROWS][4];
     __shared__ int anyfg[2];
@@ -82,30 +89,47 @@ __global__ void __launch_bounds__(PS_NT) k_psf(const __grid_constant__ PsfArgs A
         rowc[r] = make_float4(cy.b, cy.c0, cy.c1, 0.f);
         rowj[r] = make_int2(cy.i, cy.i1);
     }
-    for (int c = t; c < SC; c += PS_NT) {
-        const AxCoef cx = axis_coef(A.sb.ax, (float)mirror_idx(X0 - H + c, W));
-        colc[c] = make_float4(cx.b, cx.c0, cx.c1, 0.f);
-        colj[c] = make_int2(cx.i, cx.i1);
+    for (int q = t; q < A.nk * PS_ROWS; q += PS_NT) {
+        const int k = q / PS_ROWS, r = q - k * PS_ROWS;
+        const AxCoef cy = axis_coef(A.ct[k].ay, (float)min(Y0 + r, Hf - 1));
+        modec[k][r] = make_float4(cy.b, cy.c0, cy.c1, __int_as_float(cy.i));
     }
     if (t < PS_ROWS * 4) mbits[t >> 2][t & 3] = 0u;
     if (t < 2) anyfg[t] = 0;
     __syncthreads();
-    // ---- m over the band and its halo, one pixel per thread at a time
+    // ---- m over the band and its halo, PS_FILL rows of a column at a time
     // (consecutive threads take consecutive columns)
-    for (int p = t; p < SR * SC; p += PS_NT) {
-        const int r = p / SC, c = p - r * SC;
-        const int x = mirror_idx(X0 - H + c, W), y = mirror_idx(Y0 - H + r, Hf);
-        const float4 cc = colc[c], rc = rowc[r];
-        const int2 jx = colj[c], jy = rowj[r];
-        AxCoef cx, cy;
-        cx.i = jx.x; cx.i1 = jx.y; cx.b = cc.x; cx.c0 = cc.y; cx.c1 = cc.z;
-        cy.i = jy.x; cy.i1 = jy.y; cy.b = rc.x; cy.c0 = rc.y; cy.c1 = rc.z;
-        const float2 b0 = row_eval(A.sb, cy.i, cx), b1 = row_eval(A.sb, cy.i1, cx);
-        bool bad;
-        const float v = load_px<F32>(im, x, y, bad);
-        ms[r][c] = bad ? 0.f : v - axis_combine(cy, b0.x, b1.x, b0.y, b1.y);
-        const int ri = r - H, ci = c - H;
-        if (ri >= 0 && ri < PS_ROWS && ci >= 0 && ci < PS_COLS) bads[ri][ci] = bad ? 1 : 0;
+    constexpr int NF = (SR + PS_FILL - 1) / PS_FILL;
+    for (int p = t; p < NF * SC; p += PS_NT) {
+        const int g = p / SC, c = p - g * SC;
+        const int x = mirror_idx(X0 - H + c, W);
+        const AxCoef cx = axis_coef(A.sb.ax, (float)x);
+        float val[PS_FILL];
+        bool bad[PS_FILL];
+#pragma unroll
+        for (int j = 0; j < PS_FILL; ++j) {
+            const int r = min(g * PS_FILL + j, SR - 1);
+            val[j] = load_px<F32>(im, x, mirror_idx(Y0 - H + r, Hf), bad[j]);
+        }
+        int jc = -1;
+        float2 b0 = make_float2(0.f, 0.f), b1 = b0;
+#pragma unroll
+        for (int j = 0; j < PS_FILL; ++j) {
+            const int r = g * PS_FILL + j;
+            if (r >= SR) break;
+            const float4 rc = rowc[r];
+            const int2 jy = rowj[r];
+            if (jy.x != jc) {
+                b0 = row_eval(A.sb, jy.x, cx);
+                b1 = row_eval(A.sb, jy.y, cx);
+                jc = jy.x;
+            }
+            AxCoef cy;
+            cy.b = rc.x; cy.c0 = rc.y; cy.c1 = rc.z;
+            ms[r][c] = bad[j] ? 0.f : val[j] - axis_combine(cy, b0.x, b1.x, b0.y, b1.y);
+            const int ri = r - H, ci = c - H;
+            if (ri >= 0 && ri < PS_ROWS && ci >= 0 && ci < PS_COLS) bads[ri][ci] = bad[j] ? 1 : 0;
+        }
     }
     __syncthreads();
     // ---- the K + 1 correlations of this thread's column and rows
@@ -122,46 +146,45 @@ __global__ void __launch_bounds__(PS_NT) k_psf(const __grid_constant__ PsfArgs A
         float2 F2[PS_RPT];
 #pragma unroll
         for (int r = 0; r < PS_RPT; ++r) F2[r] = make_float2(0.f, 0.f);
-#pragma unroll UNROLL_U
+#pragma unroll 1
         for (int u = 0; u < KS; ++u) {
-            float2 w[PS_RPT + KS - 1];
+            float2 tap[KS];
+#pragma unroll
+            for (int v = 0; v < KS; ++v) tap[v] = A.taps[pr][u * KS + v];
 #pragma unroll
             for (int q = 0; q < PS_RPT + KS - 1; ++q) {
                 const float a = ms[r0 + q][col + u];
-                w[q] = make_float2(a, a);
-            }
+                const float2 w = make_float2(a, a);
+                // each row meets its taps v = 0, 1, .. in order
 #pragma unroll
-            for (int v = 0; v < KS; ++v) {
-                const float2 tap = A.taps[pr][v * KS + u];
-#pragma unroll
-                for (int r = 0; r < PS_RPT; ++r) F2[r] = psf_ffma2(tap, w[r + v], F2[r]);
+                for (int r = 0; r < PS_RPT; ++r)
+                    if (q - r >= 0 && q - r < KS) F2[r] = psf_ffma2(tap[q - r], w, F2[r]);
             }
         }
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const int k = 2 * pr + h;
             if (k > A.nk) break;
-            float F[PS_RPT];
-#pragma unroll
-            for (int r = 0; r < PS_RPT; ++r) F[r] = h ? F2[r].y : F2[r].x;
             if (k == 0) {
 #pragma unroll
-                for (int r = 0; r < PS_RPT; ++r) S[r] = F[r];
+                for (int r = 0; r < PS_RPT; ++r) S[r] = F2[r].x;
             } else {
                 const SplineTab& ct = A.ct[k - 1];
                 const AxCoef cx = axis_coef(ct.ax, (float)xq);
                 int jc = -1;
-                float u0 = 0.f, u1 = 0.f, w0 = 0.f, w1 = 0.f;
+                float2 a0 = make_float2(0.f, 0.f), a1 = a0;
 #pragma unroll
                 for (int r = 0; r < PS_RPT; ++r) {
-                    const int y = min(Y0 + r0 + r, Hf - 1);
-                    const AxCoef cy = axis_coef(ct.ay, (float)y);
-                    if (cy.i != jc) {
-                        const float2 a0 = row_eval(ct, cy.i, cx), a1 = row_eval(ct, cy.i1, cx);
-                        u0 = a0.x; w0 = a0.y; u1 = a1.x; w1 = a1.y;
-                        jc = cy.i;
+                    const float4 rc = modec[k - 1][r0 + r];
+                    const int j = __float_as_int(rc.w);
+                    if (j != jc) {
+                        a0 = row_eval(ct, j, cx);
+                        a1 = row_eval(ct, min(j + 1, ct.ay.n - 1), cx);
+                        jc = j;
                     }
-                    S[r] = fmaf(axis_combine(cy, u0, u1, w0, w1), F[r], S[r]);
+                    AxCoef cy;
+                    cy.b = rc.x; cy.c0 = rc.y; cy.c1 = rc.z;
+                    S[r] = fmaf(axis_combine(cy, a0.x, a1.x, a0.y, a1.y), h ? F2[r].y : F2[r].x, S[r]);
                 }
             }
         }
@@ -169,12 +192,22 @@ __global__ void __launch_bounds__(PS_NT) k_psf(const __grid_constant__ PsfArgs A
     // ---- threshold, map, mask bits
     const AxCoef sx = axis_coef(A.sr.ax, (float)xq);
     uint32_t* srow = A.seg;
+    int jc = -1;
+    float2 q0 = make_float2(0.f, 0.f), q1 = q0;
 #pragma unroll
     for (int r = 0; r < PS_RPT; ++r) {
         const int y = Y0 + r0 + r;
         if (!xin || y >= Hf) continue;
-        const AxCoef sy = axis_coef(A.sr.ay, (float)y);
-        const float2 q0 = row_eval(A.sr, sy.i, sx), q1 = row_eval(A.sr, sy.i1, sx);
+        // the noise map's axes are the background map's
+        const float4 rc = rowc[r0 + r + H];
+        const int2 jy = rowj[r0 + r + H];
+        if (jy.x != jc) {
+            q0 = row_eval(A.sr, jy.x, sx);
+            q1 = row_eval(A.sr, jy.y, sx);
+            jc = jy.x;
+        }
+        AxCoef sy;
+        sy.b = rc.x; sy.c0 = rc.y; sy.c1 = rc.z;
         const float kt = A.thresh * axis_combine(sy, q0.x, q1.x, q0.y, q1.y);
         const bool fg = !bads[r0 + r][col] && S[r] > kt;
         const float mv = ms[r0 + r + H][col + H];
@@ -229,7 +262,7 @@ cudaError_t launch_psf(const DetectArgs& D, const float* p0, const float* modes,
         const float* src = k == 0 ? p0 : modes + (size_t)(k - 1) * kw * kh;
         for (int v = 0; v < kh; ++v)
             for (int u = 0; u < kw; ++u) {
-                float2& t = A.taps[k / 2][(v + oy) * ks + (u + ox)];
+                float2& t = A.taps[k / 2][(u + ox) * ks + (v + oy)];
                 if (k & 1) t.y = src[v * kw + u];
                 else t.x = src[v * kw + u];
             }
