@@ -156,29 +156,16 @@ __device__ __forceinline__ void mom_fold(MomAcc& a, DF r0, DF r1, DF r2, int xs,
 }
 
 // one pixel of a run: its partial sums, the peak (first pixel in raster
-// order among equal maxima) and the saturation flag
+// order among equal maxima; a lane takes its pixels in that order) and the
+// saturation flag
 __device__ __forceinline__ void run_pixel(DF& r0, DF& r1, DF& r2, MomAcc& a, float m, int x, uint32_t L, bool sat)
 {
     const float fx = (float)x;
     df_add(r0, m);
     df_add_prod(r1, fx, m);
     df_add_prod(r2, fx * fx, m);
-    if (m > a.peak || (m == a.peak && L < a.peakL)) { a.peak = m; a.peakL = L; }
+    if (m > a.peak) { a.peak = m; a.peakL = L; }
     if (sat) a.flags |= GP_FLAG_SAT;
-}
-
-// sum of v over lanes base .. base + 2^levels - 1 into lane base (a fixed
-// tree: reproducible); lanes outside the range hold zeros
-__device__ __forceinline__ DF df_tree_sum(DF v, int levels)
-{
-    const int lane = threadIdx.x & 31;
-    for (int o = levels > 0 ? 1 << (levels - 1) : 0; o > 0; o >>= 1) {
-        DF w;
-        w.hi = __shfl_down_sync(0xffffffffu, v.hi, o);
-        w.lo = __shfl_down_sync(0xffffffffu, v.lo, o);
-        if (lane + o < 32) v = df_merge(v, w);
-    }
-    return v;
 }
 
 // float -> unsigned key with the same order (+0 and -0 equal)
@@ -193,12 +180,24 @@ __device__ __forceinline__ float fkey_inv(uint32_t k)
 }
 
 // a segment's sums over the lanes (tile rows) base .. base + 2^levels - 1,
-// complete in lane base
+// complete in lane base (a fixed tree: reproducible); lanes outside the range
+// hold zeros
 __device__ __forceinline__ void mom_rows_reduce(MomAcc& a, int levels)
 {
     const uint32_t FULL = 0xffffffffu;
-    a.s = df_tree_sum(a.s, levels); a.sx = df_tree_sum(a.sx, levels); a.sy = df_tree_sum(a.sy, levels);
-    a.sxx = df_tree_sum(a.sxx, levels); a.syy = df_tree_sum(a.syy, levels); a.sxy = df_tree_sum(a.sxy, levels);
+    const int lane = threadIdx.x & 31;
+    DF* v[6] = {&a.s, &a.sx, &a.sy, &a.sxx, &a.syy, &a.sxy};
+#pragma unroll 1
+    for (int o = levels > 0 ? 1 << (levels - 1) : 0; o > 0; o >>= 1) {
+#pragma unroll
+        for (int k = 0; k < 6; ++k) {
+            DF w;
+            w.hi = __shfl_down_sync(FULL, v[k]->hi, o);
+            w.lo = __shfl_down_sync(FULL, v[k]->lo, o);
+            w = df_merge(*v[k], w);
+            if (lane + o < 32) *v[k] = w;
+        }
+    }
     a.ux = __reduce_add_sync(FULL, a.ux); a.uy = __reduce_add_sync(FULL, a.uy);
     a.uxx = __reduce_add_sync(FULL, a.uxx); a.uyy = __reduce_add_sync(FULL, a.uyy);
     a.uxy = __reduce_add_sync(FULL, a.uxy);
@@ -319,7 +318,21 @@ __device__ __forceinline__ const DetectArgs& det_frame(const DetectArgs* __restr
     else return one;
 }
 
-// write the records of kept root r (lane-parallel or lane 0 of the warp path)
+// a final segment whose sum is not positive: the unweighted moments, in
+// float64 (rare, and kept out of the labelling kernel's instruction stream)
+__device__ __noinline__ uint32_t emit_fallback(const Comps& C, int id, double s, int ux, int uy, int uxx, int uyy,
+                                               int uxy, int npix, int x0, int y0)
+{
+    double flux;
+    double2 xy;
+    Mom2 m2;
+    uint32_t fl = 0u;
+    mom_finish(s, 0.0, 0.0, 0.0, 0.0, 0.0, ux, uy, uxx, uyy, uxy, npix, x0, y0, &flux, &xy, &m2, &fl);
+    C.flux[id] = flux; C.xy[id] = xy; C.mom2[id] = m2;
+    return fl;
+}
+
+// write the records of kept root r
 template <bool LABEL_ONLY, bool BIG>
 __device__ __forceinline__ void emit_root(const DetectArgs& A, const LabelSmem<BIG>& S, int r, int4 bb, int pbase,
                                           int cbase, int x0, int y0, const MomAcc& a)
@@ -356,12 +369,7 @@ __device__ __forceinline__ void emit_root(const DetectArgs& A, const LabelSmem<B
         // sums about the tile corner (x0, y0), finished by k_mom_finish
         comp_store_raw(A.C, id, a.s, a.sx, a.sy, a.sxx, a.syy, a.sxy);
     } else {
-        double flux;
-        double2 xy;
-        Mom2 m2;
-        mom_finish(df_value(a.s), df_value(a.sx), df_value(a.sy), df_value(a.sxx), df_value(a.syy), df_value(a.sxy),
-                   a.ux, a.uy, a.uxx, a.uyy, a.uxy, npix, x0, y0, &flux, &xy, &m2, &fl);
-        A.C.flux[id] = flux; A.C.xy[id] = xy; A.C.mom2[id] = m2;
+        fl |= emit_fallback(A.C, id, df_value(a.s), a.ux, a.uy, a.uxx, a.uyy, a.uxy, npix, x0, y0);
     }
     A.C.peak[id] = a.peak; A.C.peakL[id] = a.peakL; A.C.flags[id] = fl;
 }
@@ -377,6 +385,11 @@ __device__ __forceinline__ bool pix_sat(const DetectArgs& A, bool async, uint32_
     return v >= A.im.sat;
 }
 
+// The warps of an SM are each at another step of a long body, so the common
+// form was bound by instruction fetch (half of a warp's time, 283 us for the
+// 74,000 tiles of a crowded 12288 x 12304 frame): the sums and the emission stand
+// once, loops are not unrolled, rare float64 is out of line, and it takes
+// 175 us.  What is left is issue and the divergence of rows (14 lanes of 32).
 template <bool LABEL_ONLY, bool BATCH, bool BIG>
 __global__ void __launch_bounds__(32 * LabelCfg<BIG>::NW, BIG ? 4 : 11) k_label_tiles(const DetectArgs* __restrict__ batch,
                                                                         const __grid_constant__ DetectArgs one,
@@ -451,6 +464,7 @@ __global__ void __launch_bounds__(32 * LabelCfg<BIG>::NW, BIG ? 4 : 11) k_label_
             const int64_t rowL = (int64_t)(y0 + y) * W + x0;
             const int64_t rowI = (int64_t)(y0 + y) * A.im.pitch + x0;
             uint64_t mb = M;
+#pragma unroll 1
             for (int f = fb; mb; ++f) {
                 const int x = __ffsll((long long)mb) - 1;
                 mb &= mb - 1;
@@ -468,6 +482,7 @@ __global__ void __launch_bounds__(32 * LabelCfg<BIG>::NW, BIG ? 4 : 11) k_label_
         {
             uint64_t hb = heads;
             int f = fb;
+#pragma unroll 1
             for (int q = rb; hb; ++q) {
                 const int x = __ffsll((long long)hb) - 1;
                 hb &= hb - 1;
@@ -496,14 +511,20 @@ __global__ void __launch_bounds__(32 * LabelCfg<BIG>::NW, BIG ? 4 : 11) k_label_
             const uint64_t V = O & ~(O << 1);
             const uint64_t NWm = M & ~U & (U << 1) & ~(M << 1);
             const uint64_t NEm = M & ~U & (U >> 1) & ~(M >> 1);
-            uint64_t sites = V | NWm | NEm;
-            while (sites) {
-                const int x = __ffsll((long long)sites) - 1;
-                sites &= sites - 1;
-                const int a = rb + __popcll((long long)(heads & upto(x))) - 1;
-                if ((V >> x) & 1ull) lunite(S.par, a, ub + __popcll((long long)(uh & upto(x))) - 1);
-                if ((NWm >> x) & 1ull) lunite(S.par, a, ub + __popcll((long long)(uh & upto(x - 1))) - 1);
-                if ((NEm >> x) & 1ull) lunite(S.par, a, ub + __popcll((long long)(uh & upto(x + 1))) - 1);
+            uint64_t left = V | NWm, right = NEm;        // no column is in both V and NW
+#pragma unroll 1
+            while (left | right) {
+                const int x = __ffsll((long long)(left | right)) - 1;
+                const uint64_t bit = 1ull << x;
+                int xu = x + 1;                          // the upper run's column
+                if (left & bit) {
+                    xu = (V & bit) ? x : x - 1;
+                    left ^= bit;
+                } else {
+                    right ^= bit;
+                }
+                lunite(S.par, rb + __popcll((long long)(heads & upto(x))) - 1,
+                       ub + __popcll((long long)(uh & upto(xu))) - 1);
             }
         }
         __syncwarp();
@@ -511,8 +532,10 @@ __global__ void __launch_bounds__(32 * LabelCfg<BIG>::NW, BIG ? 4 : 11) k_label_
         // cnt first, then into par once every lane's walks are over -- a
         // halving store from a stale read can then never land on a root
         // that another lane has already written
+#pragma unroll 1
         for (int q = rb; q < rb + nr; ++q) S.cnt[q] = lfind(S.par, q);
         __syncwarp();
+#pragma unroll 1
         for (int q = rb; q < rb + nr; ++q) {
             S.par[q] = S.cnt[q];
             S.cnt[q] = 0;
@@ -521,6 +544,7 @@ __global__ void __launch_bounds__(32 * LabelCfg<BIG>::NW, BIG ? 4 : 11) k_label_
         // ---- pixels and shared-edge contact per root, one atomic per run
         {
             uint64_t hb = heads;
+#pragma unroll 1
             for (int q = rb; hb; ++q) {
                 const int x = __ffsll((long long)hb) - 1;
                 hb &= hb - 1;
@@ -536,6 +560,7 @@ __global__ void __launch_bounds__(32 * LabelCfg<BIG>::NW, BIG ? 4 : 11) k_label_
         // segments (>= minarea); local indices, map values, one id
         // reservation per kind per tile
         int np = 0, nc = 0, nk = 0;
+#pragma unroll 1
         for (int c0 = 0; c0 < NR; c0 += 32) {
             const int k = c0 + lane;
             bool piece = false, comp = false;
@@ -570,12 +595,14 @@ __global__ void __launch_bounds__(32 * LabelCfg<BIG>::NW, BIG ? 4 : 11) k_label_
         if (y < th) {
             uint32_t* srow = A.seg + (int64_t)(y0 + y) * W + x0;
             uint64_t hb = heads;
+#pragma unroll 1
             for (int q = rb; hb; ++q) {
                 const int x = __ffsll((long long)hb) - 1;
                 hb &= hb - 1;
                 const uint32_t v = (uint32_t)S.val[S.par[q]];
                 if (LABEL_ONLY && !v) continue;          // a given mask: the map is already 0 there
                 const int xe = run_end(M, x);
+#pragma unroll 1
                 for (int xx = x; xx <= xe; ++xx) srow[xx] = v;
             }
         }
@@ -608,6 +635,7 @@ __global__ void __launch_bounds__(32 * LabelCfg<BIG>::NW, BIG ? 4 : 11) k_label_
         // runs in label order), when the tile holds at least eight of them
         // (fewer leave most lanes idle; measured against 2, 4, 12 and 16)
         int nsmall = 0;
+#pragma unroll 1
         for (int c0 = 0; c0 < nk; c0 += 32) {
             const int i = c0 + lane;
             nsmall += __popc(__ballot_sync(FULL, i < nk && (S.cnt[S.klist[i]] & 0xffff) <= LANE_SEG_MAX));
@@ -617,14 +645,17 @@ __global__ void __launch_bounds__(32 * LabelCfg<BIG>::NW, BIG ? 4 : 11) k_label_
             // runs of each small kept segment, in label order: runs are taken
             // 32 at a time in id order; the lanes holding runs of one segment
             // find each other (match) and the first of them advances its count
+#pragma unroll 1
             for (int c0 = 0; c0 < nk; c0 += 32) {
                 const int i = c0 + lane;
                 if (i < nk) S.rcnt[S.klist[i]] = 0;
             }
+#pragma unroll 1
             for (int pass = 0; pass < 2; ++pass) {
                 if (pass == 1) {
                     // offsets: the segments' runs laid out in kept-root order
                     int off = 0;
+#pragma unroll 1
                     for (int c0 = 0; c0 < nk; c0 += 32) {
                         const int i = c0 + lane;
                         const int r = i < nk ? S.klist[i] : -1;
@@ -640,6 +671,7 @@ __global__ void __launch_bounds__(32 * LabelCfg<BIG>::NW, BIG ? 4 : 11) k_label_
                     }
                 }
                 __syncwarp();
+#pragma unroll 1
                 for (int c0 = 0; c0 < NR; c0 += 32) {
                     const int q = c0 + lane;
                     const int r = q < NR ? S.par[q] : -1;
@@ -655,70 +687,59 @@ __global__ void __launch_bounds__(32 * LabelCfg<BIG>::NW, BIG ? 4 : 11) k_label_
                     __syncwarp();
                 }
             }
-            for (int c0 = 0; c0 < nk; c0 += 32) {
-                const int i = c0 + lane;
-                const int r = i < nk ? S.klist[i] : -1;
-                if (r < 0 || (S.cnt[r] & 0xffff) > LANE_SEG_MAX) continue;
-                MomAcc a;
-                mom_zero(a);
-                int bx0 = TX, bx1 = -1, by1 = -1;
-                const int e0 = S.roff[r], e1 = e0 + S.rcnt[r];
-                for (int e = e0; e < e1; ++e) {
-                    const int q = S.rlist[e];
-                    const int p = S.pos[q], ry = p / TX, rx = p % TX, n = S.len[q] + 1;
-                    bx0 = min(bx0, rx); bx1 = max(bx1, rx + n - 1); by1 = ry;
-                    if (!LABEL_ONLY) {
-                        const int f0 = S.fidx[q];
-                        const int64_t lin = (int64_t)(y0 + ry) * A.im.pitch + x0 + rx;
-                        const uint32_t L0 = (uint32_t)(y0 + ry) * (uint32_t)W + (uint32_t)(x0 + rx);
-                        DF r0 = df_zero(), r1 = df_zero(), r2 = df_zero();
-                        for (int t = 0; t < n; ++t)
-                            run_pixel(r0, r1, r2, a, S.m[f0 + t], rx + t, L0 + t,
-                                      sat_on && pix_sat(A, sat_async, S.iv[f0 + t], lin + t));
-                        mom_fold(a, r0, r1, r2, rx, rx + n - 1, ry);
-                    }
-                }
-                const int ry0 = S.pos[r] / TX;
-                emit_root<LABEL_ONLY, BIG>(A, S, r, make_int4(x0 + bx0, x0 + bx1, y0 + ry0, y0 + by1), pbase, cbase,
-                                           x0, y0, a);
-            }
         }
-        // ---- the other kept segments: the whole warp, lane = tile row; the
-        // sums meet in the segment's first row by a tree over its rows
-        for (int i = 0; i < nk; ++i) {
-            const int r = S.klist[i];
-            if (lane_path && (S.cnt[r] & 0xffff) <= LANE_SEG_MAX) continue;
-            int xmin = TX, xmax = -1;
+        // ---- the segments' sums, in one loop so that its code is there once:
+        // first 32 small segments at a time, a lane each; then the others by
+        // the whole warp, lane = tile row, whose sums meet in the segment's
+        // first row by a tree over its rows
+        const int ngroup = lane_path ? (nk + 31) / 32 : 0;
+#pragma unroll 1
+        for (int i = 0; i < ngroup + nk; ++i) {
+            const bool group = i < ngroup;
+            int r = -1, e0 = rb, e1 = rb + nr;
+            if (group) {
+                if (i * 32 + lane < nk) r = S.klist[i * 32 + lane];
+                if (r >= 0 && (S.cnt[r] & 0xffff) > LANE_SEG_MAX) r = -1;
+                e0 = r >= 0 ? S.roff[r] : 0;
+                e1 = r >= 0 ? e0 + S.rcnt[r] : 0;
+            } else {
+                r = S.klist[i - ngroup];
+                if (lane_path && (S.cnt[r] & 0xffff) <= LANE_SEG_MAX) continue;
+            }
             MomAcc a;
             mom_zero(a);
-            uint64_t hb = heads;
-            for (int q = rb; hb; ++q) {
-                const int x = __ffsll((long long)hb) - 1;
-                hb &= hb - 1;
-                if (S.par[q] != r) continue;
-                const int xe = run_end(M, x);
-                xmin = min(xmin, x);
-                xmax = max(xmax, xe);
+            int bx0 = TX, bx1 = -1, by1 = -1;
+#pragma unroll 1
+            for (int e = e0; e < e1; ++e) {
+                const int q = group ? S.rlist[e] : e;
+                if (!group && S.par[q] != r) continue;
+                const int p = S.pos[q], ry = p / TX, rx = p % TX, n = S.len[q] + 1;
+                bx0 = min(bx0, rx); bx1 = max(bx1, rx + n - 1); by1 = ry;
                 if (!LABEL_ONLY) {
                     const int f0 = S.fidx[q];
-                    const int64_t lin = (int64_t)(y0 + y) * A.im.pitch + x0 + x;
-                    const uint32_t L0 = (uint32_t)(y0 + y) * (uint32_t)W + (uint32_t)(x0 + x);
+                    const int64_t lin = (int64_t)(y0 + ry) * A.im.pitch + x0 + rx;
+                    const uint32_t L0 = (uint32_t)(y0 + ry) * (uint32_t)W + (uint32_t)(x0 + rx);
                     DF r0 = df_zero(), r1 = df_zero(), r2 = df_zero();
-                    for (int t = 0; t <= xe - x; ++t)
-                        run_pixel(r0, r1, r2, a, S.m[f0 + t], x + t, L0 + t,
+#pragma unroll 1
+                    for (int t = 0; t < n; ++t)
+                        run_pixel(r0, r1, r2, a, S.m[f0 + t], rx + t, L0 + t,
                                   sat_on && pix_sat(A, sat_async, S.iv[f0 + t], lin + t));
-                    mom_fold(a, r0, r1, r2, x, xe, y);
+                    mom_fold(a, r0, r1, r2, rx, rx + n - 1, ry);
                 }
             }
-            const bool present = xmax >= 0;
-            const int ry0 = S.pos[r] / TX;
-            const int bx0 = __reduce_min_sync(FULL, xmin), bx1 = __reduce_max_sync(FULL, xmax);
-            const int by1 = __reduce_max_sync(FULL, present ? y : -1);
-            if (!LABEL_ONLY) {
-                const int span = by1 - ry0 + 1;
-                mom_rows_reduce(a, span <= 1 ? 0 : 32 - __clz(span - 1));
+            const int ry0 = r >= 0 ? S.pos[r] / TX : 0;
+            bool mine = r >= 0;
+            if (!group) {
+                bx0 = __reduce_min_sync(FULL, bx0);
+                bx1 = __reduce_max_sync(FULL, bx1);
+                by1 = __reduce_max_sync(FULL, by1);
+                if (!LABEL_ONLY) {
+                    const int span = by1 - ry0 + 1;
+                    mom_rows_reduce(a, span <= 1 ? 0 : 32 - __clz(span - 1));
+                }
+                mine = lane == ry0;
             }
-            if (lane == ry0)
+            if (mine)
                 emit_root<LABEL_ONLY, BIG>(A, S, r, make_int4(x0 + bx0, x0 + bx1, y0 + ry0, y0 + by1), pbase, cbase,
                                            x0, y0, a);
         }
