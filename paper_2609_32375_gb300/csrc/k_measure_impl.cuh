@@ -114,35 +114,46 @@ __device__ __forceinline__ float pixel_area(float dx0, float dy0, float r)
 // Pixels crossed by a circle wait in a per-warp queue so that the exact
 // overlap area, the one expensive step, runs with every lane busy instead of
 // once per row for whichever lanes meet the circle.
-struct BEntry {
-    float dx0, dy0, m, var;
-    int kf;                 // mask of the radii crossing the pixel | bad << 8 | saturated << 9
-};
 constexpr int QCAP = 64;      // at most 31 waiting + 32 added by one row
 constexpr int MEAS_NT = 256;
+
+// a row's terms, each computed by one lane: the y-spline's coefficients in
+// pairs (for the background and the noise at once), ny^2 and the larger
+// dy^2 of its edges, dy0, and its node row
+struct ApRow {
+    float4 p;               // b, b, c0, c0
+    float4 q;               // c1, c1, ny^2, max dy^2
+    float2 r;               // dy0, i
+};
+struct ApWarp {
+    ApRow row[32];
+    float4 px[QCAP];        // the queue: dx0, dy0, m, var
+    int kf[QCAP];           // mask of the radii crossing the pixel | bad << 8 | saturated << 9
+};
 
 // the flag bits a lane collects: bit k a bad pixel under disc k, bit 8 + k a
 // saturated one
 template <int NR>
-__device__ __forceinline__ void flush_queue(const ApSpec& ap, BEntry* wq, int qn, DF* f, DF* v, uint32_t& pk)
+__device__ __forceinline__ void flush_queue(const ApSpec& ap, const ApWarp* wq, int qn, DF* f, DF* v, uint32_t& pk)
 {
     __syncwarp();
     const int lane = threadIdx.x & 31;
     for (int i = lane; i < qn; i += 32) {
-        const BEntry e = wq[i];
-        unsigned rm = e.kf & 0xffu;                  // the radii whose circle crosses the pixel
+        const float4 e = wq->px[i];
+        const int kf = wq->kf[i];
+        unsigned rm = kf & 0xffu;                    // the radii whose circle crosses the pixel
         while (rm) {
             const int k = __ffs(rm) - 1;
             rm &= rm - 1u;
-            const float A = pixel_area(e.dx0, e.dy0, ap.r[k]);
+            const float A = pixel_area(e.x, e.y, ap.r[k]);
             if (!(A > 0.f)) continue;
-            if (e.kf & 0x100) { pk |= 1u << k; continue; }
-            if (e.kf & 0x200) pk |= 0x100u << k;
+            if (kf & 0x100) { pk |= 1u << k; continue; }
+            if (kf & 0x200) pk |= 0x100u << k;
 #pragma unroll
             for (int kk = 0; kk < NR; ++kk) {
                 if (kk != k) continue;
-                df_add_prod(f[kk], A, e.m);
-                df_add_prod(v[kk], A, e.var);
+                df_add_prod(f[kk], A, e.z);
+                df_add_prod(v[kk], A, e.w);
             }
         }
     }
@@ -200,16 +211,20 @@ __device__ __forceinline__ int scatter_index(int lane)
 // Apertures around (cx, cy) for all radii; executed by one full warp.
 // One lane per pixel column: the column's x-spline coefficients and the
 // node-row values u_j, w_j of both maps are evaluated once per column and
-// reused down the column; the y-spline coefficients of up to 32 rows are
-// evaluated one row per lane and fetched by shuffle, so each pixel costs a
-// few FMAs for B(p) and sigma(p).  Pixels wholly inside disc k add to a lane's
+// reused down the column; the terms of up to 32 rows are evaluated one row
+// per lane and read back from shared memory, so each pixel costs a few paired
+// FMAs for B(p) and sigma(p) together.  Pixels wholly inside disc k add to a lane's
 // float32 column sums (at most 32 terms, then folded into float-float sums);
-// pixels the circle crosses go through the queue.  The queue order and the
+// pixels the circle crosses go through the queue.  Bound by instruction issue (the integer and
+// compare pipe first): a crowded 151 MP frame's
+// rows with radii 3, 6 and 10 take 282
+// us, 326 before the rows' terms were shared, the two maps paired and
+// the pixels loaded ahead.  The queue order and the
 // lane assignment are fixed, and lane results are combined in a fixed order,
 // so the sums are reproducible.
 template <bool F32, int NR>
 __device__ void aperture_warp(const Image& im, const SplineTab& sb, const SplineTab& sr, const ApSpec& ap,
-                              double cx, double cy, double* flux, double* ferr, uint32_t* aflags, BEntry* wq)
+                              double cx, double cy, double* flux, double* ferr, uint32_t* aflags, ApWarp* wq)
 {
     const int lane = threadIdx.x & 31;
     const unsigned lt = (1u << lane) - 1u;
@@ -239,6 +254,10 @@ __device__ void aperture_warp(const Image& im, const SplineTab& sb, const Spline
     DF* v = acc + NRA;
     uint32_t pk = 0u;                                // bad (bit k) / saturated (bit 8 + k) under disc k
     const float rmax2 = ap.rmax * ap.rmax;
+    float r2[NRA];
+#pragma unroll
+    for (int k = 0; k < NR; ++k) r2[k] = ap.r[k] * ap.r[k];
+    const float satv = im.sat > 0.f ? im.sat : __int_as_float(0x7fffffff);   // NaN: no value reaches it
     const int nyn = sb.ay.n;
     int qn = 0;                                      // warp-uniform queue length
     for (int xbase = xa; xbase <= xb; xbase += 32) {
@@ -246,78 +265,104 @@ __device__ void aperture_warp(const Image& im, const SplineTab& sb, const Spline
         const bool colok = x <= xb;
         const int xl = colok ? x : xb;
         const float dx0 = (float)(x - xi) - xf - 0.5f, dx1 = dx0 + 1.f;
-        const float nx = fmaxf(0.f, fmaxf(dx0, -dx1));
-        const float fx = fmaxf(dx0 * dx0, dx1 * dx1);
+        // a lane past the window compares as NaN: in no disc
+        const float nx = colok ? fmaxf(0.f, fmaxf(dx0, -dx1)) : __int_as_float(0x7fffffff);
+        const float fx = colok ? fmaxf(dx0 * dx0, dx1 * dx1) : __int_as_float(0x7fffffff);
         const AxCoef ccx = axis_coef(sb.ax, (float)xl);
         int jc = -1;                       // node row pair cached for this column
-        float ub0 = 0, ub1 = 0, wb0 = 0, wb1 = 0, ur0 = 0, ur1 = 0, wr0 = 0, wr1 = 0;
+        // (background, noise) of the column: values, differences, second derivatives
+        unsigned long long u0 = 0, du = 0, w0 = 0, w1 = 0;
         for (int ybase = ya; ybase <= yb; ybase += 32) {
-            const AxCoef cyl = axis_coef(sb.ay, (float)min(ybase + lane, yb));   // row ybase + lane
-            const int yend = min(yb, ybase + 31);
-            float fs[NRA], vs[NRA];
-#pragma unroll
-            for (int k = 0; k < NRA; ++k) { fs[k] = 0.f; vs[k] = 0.f; }
-            for (int y = ybase; y <= yend; ++y) {
+            // the rows that meet the largest disc are consecutive
+            int jlo, jhi;
+            {
+                const int y = min(ybase + lane, yb);
+                const AxCoef c = axis_coef(sb.ay, (float)y);
                 const float dy0 = (float)(y - yi) - yf - 0.5f, dy1 = dy0 + 1.f;
                 const float ny = fmaxf(0.f, fmaxf(dy0, -dy1));
-                if (!(ny * ny < rmax2)) continue;        // a row beyond the largest disc (the whole warp)
-                const int j = y - ybase;
-                AxCoef ccy;
-                ccy.i = __shfl_sync(0xffffffffu, cyl.i, j);
-                ccy.b = __shfl_sync(0xffffffffu, cyl.b, j);
-                ccy.c0 = __shfl_sync(0xffffffffu, cyl.c0, j);
-                ccy.c1 = __shfl_sync(0xffffffffu, cyl.c1, j);
-                ccy.i1 = min(ccy.i + 1, nyn - 1);
-                if (ccy.i != jc) {
-                    const float2 b0 = row_eval(sb, ccy.i, ccx), b1 = row_eval(sb, ccy.i1, ccx);
-                    const float2 r0 = row_eval(sr, ccy.i, ccx), r1 = row_eval(sr, ccy.i1, ccx);
-                    ub0 = b0.x; wb0 = b0.y; ub1 = b1.x; wb1 = b1.y;
-                    ur0 = r0.x; wr0 = r0.y; ur1 = r1.x; wr1 = r1.y;
-                    jc = ccy.i;
+                const float ny2 = ny * ny;
+                const unsigned on = __ballot_sync(0xffffffffu, ybase + lane <= yb && ny2 < rmax2);
+                jlo = __ffs(on) - 1;
+                jhi = 31 - __clz(on);
+                __syncwarp();                        // the rows before are done with
+                wq->row[lane].p = make_float4(c.b, c.b, c.c0, c.c0);
+                wq->row[lane].q = make_float4(c.c1, c.c1, ny2, fmaxf(dy0 * dy0, dy1 * dy1));
+                wq->row[lane].r = make_float2(dy0, __int_as_float(c.i));
+                __syncwarp();
+                if (!on) continue;
+            }
+            unsigned long long fv[NRA];              // column sums of (m, variance)
+#pragma unroll
+            for (int k = 0; k < NRA; ++k) fv[k] = 0ull;
+            // pixels two rows ahead
+            bool bad1, bad2;
+            float val1 = load_px<F32>(im, xl, ybase + jlo, bad1);
+            float val2 = load_px<F32>(im, xl, ybase + min(jlo + 1, jhi), bad2);
+#pragma unroll 1
+            for (int j = jlo; j <= jhi; ++j) {
+                const float val = val1;
+                const bool bad = bad1;
+                val1 = val2;
+                bad1 = bad2;
+                val2 = load_px<F32>(im, xl, ybase + min(j + 2, jhi), bad2);
+                const float4 p = wq->row[j].p, q = wq->row[j].q;
+                const float2 r = wq->row[j].r;
+                const int i = __float_as_int(r.y);
+                if (i != jc) {
+                    const int i1 = min(i + 1, nyn - 1);
+                    const float2 b0 = row_eval(sb, i, ccx), b1 = row_eval(sb, i1, ccx);
+                    const float2 r0 = row_eval(sr, i, ccx), r1 = row_eval(sr, i1, ccx);
+                    u0 = f2pack(b0.x, r0.x);
+                    du = f2sub(f2pack(b1.x, r1.x), u0);
+                    w0 = f2pack(b0.y, r0.y);
+                    w1 = f2pack(b1.y, r1.y);
+                    jc = i;
                 }
-                const float dmin2 = fmaf(nx, nx, ny * ny);
-                const float dmax2 = fx + fmaxf(dy0 * dy0, dy1 * dy1);
-                const bool live = colok && dmin2 < rmax2;
-                bool bad;
-                const float val = load_px<F32>(im, xl, y, bad);
-                const float sg = axis_combine(ccy, ur0, ur1, wr0, wr1);
-                const float m = bad ? 0.f : __fsub_rn(val, axis_combine(ccy, ub0, ub1, wb0, wb1));
+                const float dmin2 = fmaf(nx, nx, q.z);
+                const float dmax2 = fx + q.w;
+                // axis_combine of both maps
+                const unsigned long long bs = f2fma(f2pack(q.x, q.y), w1, f2fma(f2pack(p.z, p.w), w0,
+                                                    f2fma(f2pack(p.x, p.y), du, u0)));
+                const float sg = f2hi(bs);
+                const float m = bad ? 0.f : __fsub_rn(val, f2lo(bs));
                 const float var = bad ? 0.f : __fmul_rn(sg, sg);
-                const bool sat = !bad && im.sat > 0.f && val >= im.sat;
-                unsigned fm = 0u, bm = 0u;           // radii holding the pixel whole / crossing it
+                const unsigned long long mv = f2pack(m, var);
+                const bool sat = !bad && val >= satv;
+                unsigned bm = 0u;                    // radii whose circle crosses the pixel
 #pragma unroll
                 for (int k = 0; k < NR; ++k) {
-                    const float r2 = ap.r[k] * ap.r[k];
-                    const bool full = live && dmax2 <= r2;
-                    const bool in = live && dmin2 < r2;
-                    fs[k] = __fadd_rn(fs[k], full ? m : 0.f);
-                    vs[k] = __fadd_rn(vs[k], full ? var : 0.f);
-                    fm |= full ? 1u << k : 0u;
-                    bm |= (in && !full) ? 1u << k : 0u;
+                    if (dmax2 <= r2[k]) fv[k] = f2add(fv[k], mv);
+                    else if (dmin2 < r2[k]) bm |= 1u << k;
                 }
-                pk |= bad ? fm : (sat ? fm << 8 : 0u);
+                if (bad || sat) {
+#pragma unroll
+                    for (int k = 0; k < NR; ++k)
+                        if (dmax2 <= r2[k]) pk |= bad ? 1u << k : 0x100u << k;
+                }
                 // one queue entry per crossed pixel, for all its radii
                 const bool bnd = bm != 0u;
                 const unsigned bal = __ballot_sync(0xffffffffu, bnd);
                 if (bnd) {
-                    BEntry e;
-                    e.dx0 = dx0; e.dy0 = dy0; e.m = m; e.var = var;
-                    e.kf = (int)bm | (bad ? 0x100 : 0) | (sat ? 0x200 : 0);
-                    wq[qn + __popc(bal & lt)] = e;
+                    const int at = qn + __popc(bal & lt);
+                    wq->px[at] = make_float4(dx0, r.x, m, var);
+                    wq->kf[at] = (int)bm | (bad ? 0x100 : 0) | (sat ? 0x200 : 0);
                 }
                 qn += __popc(bal);
                 if (qn >= 32) {
                     // one full round of 32 entries; the rest (< 32) moves to the front
                     flush_queue<NR>(ap, wq, 32, f, v, pk);
-                    if (lane < qn - 32) wq[lane] = wq[lane + 32];
+                    if (lane < qn - 32) {
+                        wq->px[lane] = wq->px[lane + 32];
+                        wq->kf[lane] = wq->kf[lane + 32];
+                    }
                     __syncwarp();
                     qn -= 32;
                 }
             }
 #pragma unroll
             for (int k = 0; k < NR; ++k) {
-                df_add(f[k], fs[k]);
-                df_add(v[k], vs[k]);
+                df_add(f[k], f2lo(fv[k]));
+                df_add(v[k], f2hi(fv[k]));
             }
         }
     }
@@ -388,8 +433,8 @@ __global__ void __launch_bounds__(MEAS_NT, 3) k_measure(const MeasureArgs* __res
     pdl_wait();
     pdl_release();
     const MeasureArgs& A = measure_frame<BATCH>(batch, one);
-    __shared__ BEntry queue[MEAS_NT / 32][QCAP];
-    BEntry* wq = queue[threadIdx.x >> 5];
+    __shared__ ApWarp warps[MEAS_NT / 32];
+    ApWarp* wq = warps + (threadIdx.x >> 5);
     const int wid = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int nw = (gridDim.x * blockDim.x) >> 5;
     const int ncomp = min(*A.C.count, A.C.cap);
@@ -408,8 +453,8 @@ __global__ void __launch_bounds__(MEAS_NT, 3) k_aperture(Image im, SplineTab sb,
                                                       const double* xs, const double* ys, int n, double* flux,
                                                       double* ferr, uint32_t* fl)
 {
-    __shared__ BEntry queue[MEAS_NT / 32][QCAP];
-    BEntry* wq = queue[threadIdx.x >> 5];
+    __shared__ ApWarp warps[MEAS_NT / 32];
+    ApWarp* wq = warps + (threadIdx.x >> 5);
     const int wid = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int nw = (gridDim.x * blockDim.x) >> 5;
     for (int i = wid; i < n; i += nw)
