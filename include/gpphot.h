@@ -412,6 +412,12 @@ gp_status gp_box_quantiles(gp_ctx* ctx, const gp_image* img, int32_t mesh, float
 gp_status gp_cnn_conv3x3(const void* x, int32_t n, int32_t h, int32_t w, int32_t cin_p, const void* wt,
                          const float* bias, int32_t cout_p, int32_t relu, void* y, int32_t out_f32, int32_t creal,
                          gp_stream stream);
+/* the gradient at a layer's input x from dp, the one at its pre-activation:
+ * the convolution of dp with wtd (gp_cnn_pack), bf16; with act (x itself,
+ * the ReLU output of the layer before), zero where act <= 0, so that dx is that
+ * layer's dp; act NULL: ungated */
+gp_status gp_cnn_conv3x3_dgrad(const void* dp, int32_t n, int32_t h, int32_t w, int32_t cout_p, const void* wtd,
+                               int32_t cin_p, const void* act, void* dx, gp_stream stream);
 /* dW[cout][cin][3][3] and db[cout] from the layer input x and the gradient
  * dp at its pre-activation; partial (nslot*9*cout_p*cin_p floats) and bpart
  * (nslot*cout_p floats) are scratch; the slots are summed in a fixed order. */
@@ -432,6 +438,20 @@ gp_status gp_cnn_pack(const float* W, const float* b, int32_t cin, int32_t cout,
 /* one AdamW step (decoupled weight decay, bias-corrected moments) */
 gp_status gp_cnn_adamw(float* p, const float* g, float* m, float* v, int64_t n, float lr, float beta1, float beta2,
                        float eps, float weight_decay, int32_t step, gp_stream stream);
+/* one layer's training state: master weights and biases with their AdamW
+ * moments, their gradients, and the packed forms of gp_cnn_pack */
+typedef struct {
+    float *W, *b, *mW, *vW, *mb, *vb;
+    const float *dW, *db;
+    void *wt, *wtd;
+    float* bias_p;
+    int32_t cin, cout, cin_p, cout_p;
+} gp_cnn_layer;
+/* gp_cnn_adamw of every layer's W (with weight_decay) and b (without), then
+ * gp_cnn_pack of the layer, in one launch; layers is a host array.  wt, wtd and
+ * bias_p must have been packed before: their padding is not rewritten. */
+gp_status gp_cnn_update(const gp_cnn_layer* layers, int32_t nlayer, float lr, float beta1, float beta2, float eps,
+                        float weight_decay, int32_t step, gp_stream stream);
 /* features of nframes frames from their quantiles ([nframes][5][nbox]):
  * centre c = median box median, scale s = median (q75 - q25) / 1.349,
  * feat = (q - c) / s as bf16 [nframes][nbox][16]; norm = (c, s) per frame */

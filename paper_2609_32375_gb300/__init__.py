@@ -35,6 +35,7 @@ EXPORTS = ("gp_ctx_create", "gp_ctx_destroy", "gp_last_error", "gp_ctx_sync", "g
            "gp_ctx_set_walk_limit", "gp_workspace_bytes",
            "gp_background", "gp_detect", "gp_aperture", "gp_growth", "gp_optimal_radius", "gp_detect_psf", "gp_cosmetic", "gp_deblend", "gp_extract", "gp_label_mask", "gp_background_static",
            "gp_background_learned", "gp_extract_learned", "gp_box_quantiles", "gp_cnn_conv3x3", "gp_cnn_conv3x3_wgrad",
+           "gp_cnn_conv3x3_dgrad", "gp_cnn_update",
            "gp_cnn_relu_backward", "gp_cnn_mse", "gp_cnn_pack", "gp_cnn_adamw", "gp_cnn_features", "gp_cnn_targets",
            "gp_cnn_denorm", "gp_extract_batch", "gp_server_create", "gp_server_submit", "gp_server_wait",
            "gp_server_release", "gp_server_stats", "gp_server_destroy", "gp_server_request_bytes")
@@ -85,6 +86,11 @@ class GpStats(C.Structure):
 
 class GpCnnWeights(C.Structure):
     _fields_ = [("wt", C.c_void_p * 6), ("bias", C.c_void_p * 6)]
+
+
+class GpCnnLayer(C.Structure):
+    _fields_ = [(k, C.c_void_p) for k in ("W", "b", "mW", "vW", "mb", "vb", "dW", "db", "wt", "wtd", "bias_p")] + \
+               [(k, C.c_int32) for k in ("cin", "cout", "cin_p", "cout_p")]
 
 
 class GpApParams(C.Structure):
@@ -232,6 +238,8 @@ def load_library():
         L.gp_cnn_mse.argtypes = [vp, vp, i64, i32, vp, vp, i32, vp, vp]
         L.gp_cnn_pack.argtypes = [vp, vp, i32, i32, i32, i32, vp, vp, vp, vp]
         L.gp_cnn_adamw.argtypes = [vp, vp, vp, vp, i64, f, f, f, f, f, i32, vp]
+        L.gp_cnn_conv3x3_dgrad.argtypes = [vp, i32, i32, i32, i32, vp, i32, vp, vp, vp]
+        L.gp_cnn_update.argtypes = [C.POINTER(GpCnnLayer), i32, f, f, f, f, f, i32, vp]
         L.gp_cnn_features.argtypes = [vp, i32, i32, vp, vp, vp]
         L.gp_cnn_targets.argtypes = [vp, vp, vp, i32, i32, vp, vp]
         L.gp_cnn_denorm.argtypes = [vp, vp, i32, i32, vp, vp, vp]
@@ -251,7 +259,7 @@ def load_library():
             getattr(L, name).restype = st
         for name in ("gp_background_learned", "gp_extract_learned", "gp_box_quantiles", "gp_cnn_conv3x3", "gp_cnn_conv3x3_wgrad",
                      "gp_cnn_relu_backward", "gp_cnn_mse", "gp_cnn_pack", "gp_cnn_adamw", "gp_cnn_features",
-                     "gp_cnn_targets", "gp_cnn_denorm"):
+                     "gp_cnn_targets", "gp_cnn_denorm", "gp_cnn_conv3x3_dgrad", "gp_cnn_update"):
             getattr(L, name).restype = st
         _lib = L
         return L

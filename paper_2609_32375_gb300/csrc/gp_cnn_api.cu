@@ -43,7 +43,16 @@ gp_status gp_cnn_conv3x3(const void* x, int32_t n, int32_t h, int32_t w, int32_t
     if (!x || !wt || !bias || !y || n < 1 || h < 1 || w < 1) return err(GP_ERR_INVALID_ARG, "conv3x3: bad argument");
     if (!cnn_pair_supported(cin_p, cout_p)) return err(GP_ERR_INVALID_ARG, "conv3x3: unsupported channel pair");
     if (out_f32 && (creal < 1 || creal > cout_p)) return err(GP_ERR_INVALID_ARG, "conv3x3: creal out of range");
-    GP_CK(launch_cnn_conv(x, n, h, w, cin_p, wt, bias, cout_p, relu, y, out_f32, creal, S(stream)));
+    GP_CK(launch_cnn_conv(x, n, h, w, cin_p, wt, bias, cout_p, relu, y, out_f32, creal, nullptr, S(stream)));
+    return GP_OK;
+}
+
+gp_status gp_cnn_conv3x3_dgrad(const void* dp, int32_t n, int32_t h, int32_t w, int32_t cout_p, const void* wtd,
+                               int32_t cin_p, const void* act, void* dx, gp_stream stream)
+{
+    if (!dp || !wtd || !dx || n < 1 || h < 1 || w < 1) return err(GP_ERR_INVALID_ARG, "dgrad: bad argument");
+    if (!cnn_pair_supported(cout_p, cin_p)) return err(GP_ERR_INVALID_ARG, "dgrad: unsupported channel pair");
+    GP_CK(launch_cnn_conv(dp, n, h, w, cout_p, wtd, nullptr, cin_p, 0, dx, 0, 0, act, S(stream)));
     return GP_OK;
 }
 
@@ -89,6 +98,20 @@ gp_status gp_cnn_adamw(float* p, const float* g, float* m, float* v, int64_t n, 
 {
     if (!p || !g || !m || !v || n < 0 || step < 1) return err(GP_ERR_INVALID_ARG, "adamw: bad argument");
     GP_CK(launch_cnn_adamw(p, g, m, v, n, lr, beta1, beta2, eps, weight_decay, step, S(stream)));
+    return GP_OK;
+}
+
+gp_status gp_cnn_update(const gp_cnn_layer* layers, int32_t nlayer, float lr, float beta1, float beta2, float eps,
+                        float weight_decay, int32_t step, gp_stream stream)
+{
+    if (!layers || nlayer < 1 || step < 1) return err(GP_ERR_INVALID_ARG, "update: bad argument");
+    for (int l = 0; l < nlayer; ++l) {
+        const gp_cnn_layer& a = layers[l];
+        if (!a.W || !a.b || !a.mW || !a.vW || !a.mb || !a.vb || !a.dW || !a.db || !a.wt || !a.wtd || !a.bias_p ||
+            a.cin < 1 || a.cout < 1 || a.cin > a.cin_p || a.cout > a.cout_p || a.cin_p > 4096 || a.cout_p > 4096)
+            return err(GP_ERR_INVALID_ARG, "update: bad layer");
+    }
+    GP_CK(launch_cnn_update(layers, nlayer, lr, beta1, beta2, eps, weight_decay, step, S(stream)));
     return GP_OK;
 }
 

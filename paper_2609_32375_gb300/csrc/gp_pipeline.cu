@@ -225,7 +225,7 @@ gp_status run_network(Exec& ex, const gp_cnn_weights* net, const float* quant, i
         const bool last = l == GP_CNN_LAYERS - 1;
         void* o = last ? (void*)out : (void*)((l & 1) ? a1 : a0);
         PL_CUDA(launch_cnn_conv(in, nf, My, Mx, CNN_CIN_P[l], net->wt[l], net->bias[l], CNN_COUT_P[l], last ? 0 : 1,
-                                o, last ? 1 : 0, 2, ex.st));
+                                o, last ? 1 : 0, 2, nullptr, ex.st));
         in = o;
     }
     for (int f = 0; f < nf; ++f)

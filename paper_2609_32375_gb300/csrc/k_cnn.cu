@@ -75,6 +75,13 @@ __device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_grou
 template <int N>
 __device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
+// a pair of bf16 gradients where the pair of activations y is positive (sign
+// clear, not zero, not NaN), else 0
+__device__ __forceinline__ uint32_t relu_gate(uint32_t y, uint32_t d)
+{
+    return (((y & 0xffffu) - 1u < 0x7f80u) ? d & 0xffffu : 0u) | (((y >> 16) - 1u < 0x7f80u) ? d & 0xffff0000u : 0u);
+}
+
 constexpr int CONV_TX = 64;      // output positions of a tile, along a row
 
 // Rows of bf16 operands are staged 8 elements longer than they are: for 16,
@@ -105,7 +112,7 @@ struct ConvCfg {
 template <int CIP, int COP, int ROWS>
 __global__ void __launch_bounds__(ConvCfg<CIP, COP, ROWS>::NT)
 k_conv3x3(const bf16* __restrict__ x, const bf16* __restrict__ wt, const float* __restrict__ bias,
-          void* __restrict__ y, int N, int H, int W, int relu, int out_f32, int creal)
+          void* __restrict__ y, int N, int H, int W, int relu, int out_f32, int creal, const bf16* __restrict__ gate)
 {
     pdl_wait();
     pdl_release();
@@ -178,8 +185,9 @@ k_conv3x3(const bf16* __restrict__ x, const bf16* __restrict__ wt, const float* 
             for (int j = 0; j < COP / 8; ++j) {
                 const int co = j * 8 + 2 * t;
                 const float* c = acc[m][j];
-                float v0 = c[0] + bias[co], v1 = c[1] + bias[co + 1];
-                float v2 = c[2] + bias[co], v3 = c[3] + bias[co + 1];
+                const float b0 = bias ? bias[co] : 0.f, b1 = bias ? bias[co + 1] : 0.f;
+                float v0 = c[0] + b0, v1 = c[1] + b1;
+                float v2 = c[2] + b0, v3 = c[3] + b1;
                 if (relu) { v0 = fmaxf(v0, 0.f); v1 = fmaxf(v1, 0.f); v2 = fmaxf(v2, 0.f); v3 = fmaxf(v3, 0.f); }
                 if (out_f32) {
                     float* yo = reinterpret_cast<float*>(y);
@@ -195,12 +203,11 @@ k_conv3x3(const bf16* __restrict__ x, const bf16* __restrict__ wt, const float* 
                     }
                 } else {
                     bf16* yo = reinterpret_cast<bf16*>(y);
-                    if (gxa < W)
-                        *reinterpret_cast<uint32_t*>(yo + (((int64_t)n * H + row) * W + gxa) * COP + co) =
-                            pack2(__float2bfloat16_rn(v0), __float2bfloat16_rn(v1));
-                    if (gxb < W)
-                        *reinterpret_cast<uint32_t*>(yo + (((int64_t)n * H + row) * W + gxb) * COP + co) =
-                            pack2(__float2bfloat16_rn(v2), __float2bfloat16_rn(v3));
+                    const int64_t oa = (((int64_t)n * H + row) * W + gxa) * COP + co, ob = oa + 8 * COP;
+                    const uint32_t pa = pack2(__float2bfloat16_rn(v0), __float2bfloat16_rn(v1));
+                    const uint32_t pb = pack2(__float2bfloat16_rn(v2), __float2bfloat16_rn(v3));
+                    if (gxa < W) *reinterpret_cast<uint32_t*>(yo + oa) = gate ? relu_gate(ld_u32(gate + oa), pa) : pa;
+                    if (gxb < W) *reinterpret_cast<uint32_t*>(yo + ob) = gate ? relu_gate(ld_u32(gate + ob), pb) : pb;
                 }
             }
         }
@@ -212,8 +219,10 @@ k_conv3x3(const bf16* __restrict__ x, const bf16* __restrict__ wt, const float* 
 // Block (slot, dy): output rows r = slot, slot + nslot, ... of the N*H; a warp
 // for each of the three taps (dy, dx) and each 16 output channels.  Bound by
 // the mma.sync rate (about 5 cycles an SM for each m16n8k16, as in k_conv3x3)
-// on the 40 SMs that hold two of the 192 blocks: the caller chooses nslot.
-// 131,072 positions, 48 to 48 channels: 48 us; one warp a tap 53, element-wise
+// of the fullest SM: the caller chooses nslot, and with 152 (three blocks on
+// every SM) the six layers and their reductions take 156 us, with 128 178, and with 64
+// (two blocks on 40 SMs, one on the others) 235.
+// 131,072 positions, 48 to 48 channels, 64 slots: 48 us; one warp a tap 53, element-wise
 // transposed staging with a block a tap, which this replaced, 270.
 // GEMM per 64 positions of a row: M = COP
 // output channels, N = CIP input channels, K = positions.  dP and the input
@@ -331,34 +340,42 @@ __global__ void __launch_bounds__(6 * COP) k_wgrad(const bf16* __restrict__ x, c
     }
 }
 
-// dW[co][ci][3][3] (real channels) = sum over slots in slot order, a thread
-// per element of the partials' own layout (consecutive threads read
-// consecutive addresses; the writes scatter); the last block sums the bias,
+// dW[co][ci][3][3] (real channels) = sum over the slots in a fixed order, in
+// the partials' own layout (the writes scatter); the last blocks sum the bias,
 // whose partials k_wgrad makes from the dP it has staged (a kernel of its own
-// with one position a step took 287 us of a layer's step, this 7).
-__global__ void k_wgrad_reduce(const float* __restrict__ partial, const float* __restrict__ bpart, int nslot, int cip,
-                               int cop, int cir, int cor, float* __restrict__ dw, float* __restrict__ db)
+// with one position a step took 287 us of a layer's step, this 5).
+// A warp takes every WR_PARTS-th slot of 32 outputs (the partials are read in
+// 128-byte rows), and the warps' sums are added in order.
+constexpr int WR_PARTS = 8;
+__global__ void __launch_bounds__(32 * WR_PARTS)
+k_wgrad_reduce(const float* __restrict__ partial, const float* __restrict__ bpart, int nslot, int cip, int cop, int cir,
+               int cor, float* __restrict__ dw, float* __restrict__ db)
 {
     pdl_wait();
     pdl_release();
-    if (blockIdx.x == gridDim.x - 1) {
-        for (int co = threadIdx.x; co < cor; co += blockDim.x) {
-            float s = 0.f;
-#pragma unroll 16
-            for (int k = 0; k < nslot; ++k) s += bpart[k * cop + co];
-            db[co] = s;
-        }
+    __shared__ float part[WR_PARTS][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int per = 9 * cop * cip, nb = (per + 31) / 32;
+    const bool isb = (int)blockIdx.x >= nb;                          // the bias gradients follow the weights'
+    const int i = ((int)blockIdx.x - (isb ? nb : 0)) * 32 + lane, n = isb ? cop : per;
+    const float* src = isb ? bpart : partial;
+    float s = 0.f;
+    if (i < n) {
+#pragma unroll 8
+        for (int k = warp; k < nslot; k += WR_PARTS) s += src[(int64_t)k * n + i];
+    }
+    part[warp][lane] = s;
+    __syncthreads();
+    if (warp || i >= n) return;
+    s = part[0][lane];
+#pragma unroll
+    for (int p = 1; p < WR_PARTS; ++p) s += part[p][lane];
+    if (isb) {
+        if (i < cor) db[i] = s;
         return;
     }
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    const int per = 9 * cop * cip;
-    if (i >= per) return;
     const int tap = i / (cop * cip), rem = i - tap * cop * cip, co = rem / cip, ci = rem - co * cip;
-    if (co >= cor || ci >= cir) return;
-    float s = 0.f;
-#pragma unroll 16
-    for (int k = 0; k < nslot; ++k) s += partial[(int64_t)k * per + i];
-    dw[(co * cir + ci) * 9 + tap] = s;
+    if (co < cor && ci < cir) dw[(co * cir + ci) * 9 + tap] = s;
 }
 
 // -------------------------------------------------------- elementwise ---
@@ -370,15 +387,12 @@ __global__ void k_relu_backward(const bf16* __restrict__ dy, const bf16* __restr
     pdl_wait();
     pdl_release();
     const int64_t i0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
-    // y > 0 for a bf16: sign clear, not zero, not NaN
-    auto pos = [](uint32_t v) { return v - 1u < 0x7f80u; };
     for (int64_t i = i0; i < nvec; i += step) {
         const uint4 a = reinterpret_cast<const uint4*>(dy)[i], b = reinterpret_cast<const uint4*>(y)[i];
         const uint32_t av[4] = {a.x, a.y, a.z, a.w}, bv[4] = {b.x, b.y, b.z, b.w};
         uint32_t o[4];
 #pragma unroll
-        for (int e = 0; e < 4; ++e)
-            o[e] = (pos(bv[e] & 0xffffu) ? av[e] & 0xffffu : 0u) | (pos(bv[e] >> 16) ? av[e] & 0xffff0000u : 0u);
+        for (int e = 0; e < 4; ++e) o[e] = relu_gate(bv[e], av[e]);
         reinterpret_cast<uint4*>(dp)[i] = make_uint4(o[0], o[1], o[2], o[3]);
     }
     for (int64_t i = 8 * nvec + i0; i < count; i += step)
@@ -445,21 +459,60 @@ __global__ void k_pack(const float* __restrict__ W, const float* __restrict__ b,
     if (i < cop) bias_p[i] = i < cor ? b[i] : 0.f;
 }
 
+struct AdamW {
+    float lr, b1, b2, eps, c1, c2;       // c1, c2: the bias corrections 1 - beta^step
+};
+
+// one value's step
+__device__ __forceinline__ float adamw_step(const AdamW& o, float wd, float p, float g, float& m, float& v)
+{
+    m = o.b1 * m + (1.f - o.b1) * g;
+    v = o.b2 * v + (1.f - o.b2) * g * g;
+    const float mh = m / o.c1, vh = v / o.c2;
+    return p - o.lr * (mh / (sqrtf(vh) + o.eps) + wd * p);
+}
+
 __global__ void k_adamw(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m,
-                        float* __restrict__ v, int64_t n, float lr, float b1, float b2, float eps, float wd, float c1,
-                        float c2)
+                        float* __restrict__ v, int64_t n, const __grid_constant__ AdamW o, float wd)
 {
     pdl_wait();
     pdl_release();
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const float gi = g[i];
-        const float mi = b1 * m[i] + (1.f - b1) * gi;
-        const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
+        float mi = m[i], vi = v[i];
+        p[i] = adamw_step(o, wd, p[i], g[i], mi, vi);
         m[i] = mi;
         v[i] = vi;
-        const float mh = mi / c1, vh = vi / c2;
-        p[i] -= lr * (mh / (sqrtf(vh) + eps) + wd * p[i]);
     }
+}
+
+// AdamW of every layer's weights and biases and their packed forms, in one
+// launch: layer blockIdx.y, a thread a weight, the biases in the last block.
+// (Zeros beside the layer's own channels stay as k_pack left them.)  A step of the
+// six-layer network: 4 us, 62 as twelve k_adamw and six k_pack.
+__global__ void k_update(const __grid_constant__ CnnLayers L, const __grid_constant__ AdamW o, float wd)
+{
+    pdl_wait();
+    pdl_release();
+    const gp_cnn_layer& A = L.l[blockIdx.y];
+    const int cir = A.cin, cor = A.cout, n = cor * cir * 9;
+    if (blockIdx.x == gridDim.x - 1) {
+        for (int i = threadIdx.x; i < cor; i += blockDim.x) {
+            float mi = A.mb[i], vi = A.vb[i];
+            const float p = adamw_step(o, 0.f, A.b[i], A.db[i], mi, vi);
+            A.mb[i] = mi; A.vb[i] = vi; A.b[i] = p;
+            A.bias_p[i] = p;
+        }
+        return;
+    }
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    float mi = A.mW[i], vi = A.vW[i];
+    const float p = adamw_step(o, wd, A.W[i], A.dW[i], mi, vi);
+    A.mW[i] = mi; A.vW[i] = vi; A.W[i] = p;
+    const int tap = i % 9, cc = i / 9, co = cc / cir, ci = cc - co * cir;
+    const bf16 q = __float2bfloat16_rn(p);
+    reinterpret_cast<bf16*>(A.wt)[(int64_t)co * 9 * A.cin_p + tap * A.cin_p + ci] = q;
+    reinterpret_cast<bf16*>(A.wtd)[(int64_t)ci * 9 * A.cout_p + (8 - tap) * A.cout_p + co] = q;
 }
 
 // ------------------------------------------------------------ features ---
@@ -556,27 +609,27 @@ __global__ void k_targets(const float* __restrict__ bkg, const float* __restrict
 // --------------------------------------------------------------- launchers ---
 template <int CIP, int COP, int ROWS>
 static cudaError_t conv_launch_rows(const void* x, int n, int h, int w, const void* wt, const float* bias, int relu,
-                                    void* y, int out_f32, int creal, int64_t most, cudaStream_t st)
+                                    void* y, int out_f32, int creal, const void* gate, int64_t most, cudaStream_t st)
 {
     using Cfg = ConvCfg<CIP, COP, ROWS>;
     cudaFuncSetAttribute(k_conv3x3<CIP, COP, ROWS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::smem);
     const int64_t ntile = (int64_t)n * ((h + ROWS - 1) / ROWS) * ((w + CONV_TX - 1) / CONV_TX);
     launch_dep(k_conv3x3<CIP, COP, ROWS>, dim3((int)(ntile < most ? ntile : most)), dim3(Cfg::NT), Cfg::smem, st,
                reinterpret_cast<const bf16*>(x), reinterpret_cast<const bf16*>(wt), bias, y, n, h, w, relu, out_f32,
-               creal);
+               creal, reinterpret_cast<const bf16*>(gate));
     return cudaGetLastError();
 }
 
 template <int CIP, int COP>
 static cudaError_t conv_launch(const void* x, int n, int h, int w, const void* wt, const float* bias, int relu,
-                               void* y, int out_f32, int creal, cudaStream_t st)
+                               void* y, int out_f32, int creal, const void* gate, cudaStream_t st)
 {
     if (n <= 0 || h <= 0 || w <= 0) return cudaErrorInvalidConfiguration;
     // four-row tiles once there is one for every SM; below, single rows
     const int64_t tiles4 = (int64_t)n * ((h + 3) / 4) * ((w + CONV_TX - 1) / CONV_TX);
     if (tiles4 >= 152)
-        return conv_launch_rows<CIP, COP, 4>(x, n, h, w, wt, bias, relu, y, out_f32, creal, 152 * 2, st);
-    return conv_launch_rows<CIP, COP, 1>(x, n, h, w, wt, bias, relu, y, out_f32, creal, 152 * 8, st);
+        return conv_launch_rows<CIP, COP, 4>(x, n, h, w, wt, bias, relu, y, out_f32, creal, gate, 152 * 2, st);
+    return conv_launch_rows<CIP, COP, 1>(x, n, h, w, wt, bias, relu, y, out_f32, creal, gate, 152 * 8, st);
 }
 
 template <int CIP, int COP>
@@ -603,9 +656,9 @@ bool cnn_pair_supported(int cip, int cop)
 }
 
 cudaError_t launch_cnn_conv(const void* x, int n, int h, int w, int cip, const void* wt, const float* bias, int cop,
-                            int relu, void* y, int out_f32, int creal, cudaStream_t st)
+                            int relu, void* y, int out_f32, int creal, const void* gate, cudaStream_t st)
 {
-#define GP_P(a, b) if (cip == a && cop == b) return conv_launch<a, b>(x, n, h, w, wt, bias, relu, y, out_f32, creal, st);
+#define GP_P(a, b) if (cip == a && cop == b) return conv_launch<a, b>(x, n, h, w, wt, bias, relu, y, out_f32, creal, gate, st);
     GP_CNN_PAIRS(GP_P)
 #undef GP_P
     return cudaErrorInvalidValue;
@@ -619,7 +672,7 @@ cudaError_t launch_cnn_wgrad(const void* x, const void* dp, int n, int h, int w,
     GP_CNN_PAIRS(GP_P)
 #undef GP_P
     if (e != cudaSuccess) return e;
-    launch_dep(k_wgrad_reduce, dim3((9 * cop * cip + 255) / 256 + 1), dim3(256), 0, st, partial, bpart, nslot, cip,
+    launch_dep(k_wgrad_reduce, dim3((9 * cop * cip + 31) / 32 + (cop + 31) / 32), dim3(32 * WR_PARTS), 0, st, partial, bpart, nslot, cip,
                cop, cir, cor, dw, db);
     return cudaGetLastError();
 }
@@ -649,11 +702,32 @@ cudaError_t launch_cnn_pack(const float* W, const float* b, int cir, int cor, in
     return cudaGetLastError();
 }
 
+static AdamW adamw_of(float lr, float b1, float b2, float eps, int step)
+{
+    return {lr, b1, b2, eps, 1.f - powf(b1, (float)step), 1.f - powf(b2, (float)step)};
+}
+
 cudaError_t launch_cnn_adamw(float* p, const float* g, float* m, float* v, int64_t n, float lr, float b1, float b2,
                              float eps, float wd, int step, cudaStream_t st)
 {
-    const float c1 = 1.f - powf(b1, (float)step), c2 = 1.f - powf(b2, (float)step);
-    launch_dep(k_adamw, dim3(152 * 2), dim3(256), 0, st, p, g, m, v, n, lr, b1, b2, eps, wd, c1, c2);
+    launch_dep(k_adamw, dim3(152 * 2), dim3(256), 0, st, p, g, m, v, n, adamw_of(lr, b1, b2, eps, step), wd);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_cnn_update(const gp_cnn_layer* layers, int nlayer, float lr, float b1, float b2, float eps, float wd,
+                              int step, cudaStream_t st)
+{
+    for (int l0 = 0; l0 < nlayer; l0 += CNN_LAYERS) {
+        CnnLayers L = {};
+        const int k = nlayer - l0 < CNN_LAYERS ? nlayer - l0 : CNN_LAYERS;
+        int most = 0;
+        for (int l = 0; l < k; ++l) {
+            L.l[l] = layers[l0 + l];
+            const int n = L.l[l].cin * L.l[l].cout * 9;
+            most = n > most ? n : most;
+        }
+        launch_dep(k_update, dim3((most + 255) / 256 + 1, k), dim3(256), 0, st, L, adamw_of(lr, b1, b2, eps, step), wd);
+    }
     return cudaGetLastError();
 }
 

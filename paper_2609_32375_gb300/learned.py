@@ -22,12 +22,12 @@ from dataclasses import dataclass
 
 import numpy as np
 
-from . import (GP_OK, GpBkg, GpBkgParams, GpCnnWeights, GpError, _check, load_library, make_image)
+from . import (GP_OK, GpBkg, GpBkgParams, GpCnnLayer, GpCnnWeights, GpError, _check, load_library, make_image)
 
 ARCH = (5, 32, 48, 48, 32, 32, 2)
 CIP = (16, 32, 48, 48, 32, 32)      # padded input channels per layer
 COP = (32, 48, 48, 32, 32, 16)      # padded output channels per layer
-NSLOT = 64                          # weight-gradient partial slots
+NSLOT = 152                         # weight-gradient partial slots (three blocks each, and on every SM)
 _STATE_LISTS = ("W", "b", "mW", "vW", "mb", "vb")   # per-layer tensors of the training state
 
 
@@ -100,6 +100,7 @@ class Network:
         N, H, Wd, _ = feat.shape
         acts = [feat]
         x = feat
+        st = _s(stream)
         for l in range(6):
             last = l == 5
             if last:
@@ -108,7 +109,7 @@ class Network:
                 y = torch.empty((N, H, Wd, COP[l]), dtype=torch.bfloat16, device=self.device)
             _check(self._lib.gp_cnn_conv3x3(x.data_ptr(), N, H, Wd, CIP[l], self.wt[l].data_ptr(),
                                             self.bias[l].data_ptr(), COP[l], 0 if last else 1, y.data_ptr(),
-                                            1 if last else 0, 2, _s(stream)))
+                                            1 if last else 0, 2, st))
             if not last:
                 acts.append(y)
             x = y
@@ -130,38 +131,31 @@ class Network:
         maxw = max(COP[l] * CIP[l] for l in range(6))
         partial = torch.empty(NSLOT * 9 * maxw, dtype=torch.float32, device=self.device)
         bpart = torch.empty(NSLOT * 64, dtype=torch.float32, device=self.device)
+        st = _s(stream)
+        dp = dy                 # the gradient at layer l's pre-activation
         for l in range(5, -1, -1):
-            if l == 5:
-                dp = dy
-            else:
-                dp = torch.empty_like(acts[l + 1])
-                _check(self._lib.gp_cnn_relu_backward(dy.data_ptr(), acts[l + 1].data_ptr(), dp.data_ptr(),
-                                                      dp.numel(), _s(stream)))
             dW = torch.empty((ARCH[l + 1], ARCH[l], 3, 3), dtype=torch.float32, device=self.device)
             db = torch.empty(ARCH[l + 1], dtype=torch.float32, device=self.device)
             _check(self._lib.gp_cnn_conv3x3_wgrad(acts[l].data_ptr(), dp.data_ptr(), N, H, Wd, CIP[l], COP[l],
                                                   ARCH[l], ARCH[l + 1], NSLOT, partial.data_ptr(),
-                                                  bpart.data_ptr(), dW.data_ptr(), db.data_ptr(), _s(stream)))
+                                                  bpart.data_ptr(), dW.data_ptr(), db.data_ptr(), st))
             grads[l] = (dW, db)
             if l > 0:
                 dx = torch.empty((N, H, Wd, CIP[l]), dtype=torch.bfloat16, device=self.device)
-                zero = torch.zeros(CIP[l], dtype=torch.float32, device=self.device)
-                _check(self._lib.gp_cnn_conv3x3(dp.data_ptr(), N, H, Wd, COP[l], self.wtd[l].data_ptr(),
-                                                zero.data_ptr(), CIP[l], 0, dx.data_ptr(), 0, 0, _s(stream)))
-                dy = dx
+                _check(self._lib.gp_cnn_conv3x3_dgrad(dp.data_ptr(), N, H, Wd, COP[l], self.wtd[l].data_ptr(), CIP[l],
+                                                      acts[l].data_ptr(), dx.data_ptr(), st))
+                dp = dx
         return loss, grads
 
     def adamw(self, grads, lr=2e-3, betas=(0.9, 0.999), eps=1e-8, wd=1e-4, stream=None):
         self.step += 1
+        layers = (GpCnnLayer * 6)()
         for l in range(6):
             dW, db = grads[l]
-            _check(self._lib.gp_cnn_adamw(self.W[l].data_ptr(), dW.data_ptr(), self.mW[l].data_ptr(),
-                                          self.vW[l].data_ptr(), self.W[l].numel(), lr, betas[0], betas[1], eps, wd,
-                                          self.step, _s(stream)))
-            _check(self._lib.gp_cnn_adamw(self.b[l].data_ptr(), db.data_ptr(), self.mb[l].data_ptr(),
-                                          self.vb[l].data_ptr(), self.b[l].numel(), lr, betas[0], betas[1], eps, 0.0,
-                                          self.step, _s(stream)))
-        self.pack(stream)
+            layers[l] = GpCnnLayer(*(t.data_ptr() for t in (
+                self.W[l], self.b[l], self.mW[l], self.vW[l], self.mb[l], self.vb[l], dW, db, self.wt[l], self.wtd[l],
+                self.bias[l])), ARCH[l], ARCH[l + 1], CIP[l], COP[l])
+        _check(self._lib.gp_cnn_update(layers, 6, lr, betas[0], betas[1], eps, wd, self.step, _s(stream)))
 
     def train_step(self, feat, target, lr=2e-3, stream=None):
         acts, out = self.forward(feat, stream)
