@@ -1511,8 +1511,8 @@ __global__ void k_bkg_maps(SplineTab sb, SplineTab sr, int W, int H, float* bmap
 // FMAs only.  FP32 throughout: the tables are stored in FP32 anyway, and the
 // diagonally dominant spline system loses nothing that matters at 1e-5.
 // Bound by latency, a line's recurrences above all: the lines' values are
-// loaded SL_AHEAD nodes ahead of them.  A 2048 x 2048 frame's 32 x 32 mesh
-// takes 7.5 us and a 64 x 64 one 17.6 (13 and 34 with both maps in one CTA, a
+// loaded SL_AHEAD nodes ahead of them.  A 16 x 16 mesh
+// takes 7.5 us and a 48 x 49 one 17.6 (13 and 34 with both maps in one CTA, a
 // load before each step and every pivot divided out).
 constexpr int MESH_SMEM_NODES = 4096;
 constexpr int MA_NT = 1024;
