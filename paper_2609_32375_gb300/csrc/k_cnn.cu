@@ -12,15 +12,16 @@
 // in float32.
 //
 //  k_conv3x3   implicit GEMM on the tensor cores (mma.sync m16n8k16 bf16):
-//              one CTA per 64 output positions of one row, the 3-row input
-//              patch and the whole weight matrix staged in shared memory.
+//              one CTA per 64 output positions of four rows or of one, the
+//              input patch and the whole weight matrix staged in shared memory.
 //              Also computes the data gradient (with flipped, transposed
-//              weights).
+//              weights), gated by the layer's ReLU as it is stored.
 //  k_wgrad     weight gradient dW[co][tap][ci] = sum_p dP[p][co] x[p+tap][ci]
 //              as a tensor-core GEMM over positions, one partial per slot,
 //              slots summed in a fixed order (reproducible).
-//  others      ReLU backward, MSE loss, weight packing, AdamW, features,
-//              output denormalisation.
+//  k_update    AdamW of all layers and the packing of their weights.
+//  others      ReLU backward, MSE loss, features, output denormalisation, and
+//              packing and AdamW of one layer.
 #include <cuda_bf16.h>
 #include <math.h>
 
