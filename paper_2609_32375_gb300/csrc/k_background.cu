@@ -178,12 +178,26 @@ struct FullHist {
     __device__ uint32_t select(unsigned long long r) { return hist_select(hist, pc, r); }
 };
 
+// The integer bounds [x, y] of med -/+ k sigma in float64, with sigma =
+// sqrt(num) / n (out of line: few boxes need it)
+__device__ __noinline__ uint2 clip_bounds_f64(uint32_t m0, uint32_t m1, unsigned long long num, unsigned long long n,
+                                              double k, uint32_t a, uint32_t b)
+{
+    const double med = 0.5 * ((double)m0 + (double)m1);
+    const double sd = sqrt_pos((double)num) * recip_pos((double)n);
+    const double ca = ceil(med - k * sd), cb = floor(med + k * sd);
+    return make_uint2(ca <= (double)a ? a : (uint32_t)ca, cb >= (double)b ? b : (cb < 0 ? 0u : (uint32_t)cb));
+}
+
 // Iterative k-sigma clip about the median on a histogram (one full warp):
 // the kept set is always the values in an integer range [a, b]; statistics
-// from exact integer sums, median by rank selection.  The passes' bounds come
-// from a float-float sigma (46 bits, and exact where the root and quotient
-// are): a float64 warp instruction holds this GPU's SM for 16 cycles, and the
-// chain of a pass held some 30.  The final statistics are float64.
+// from exact integer sums, median by rank selection.  A float64 warp
+// instruction holds this GPU's SM for 16 cycles, and the chain of a pass held
+// some 30, so a pass first takes its bounds in float-float, whose error is
+// below 2^-44 of their terms.  Only the integer beyond a bound matters: unless
+// an integer lies within 2^-40 of the bound (a tie, as two-valued boxes make
+// them), float64 would name the same one; then float64 decides.  The final
+// statistics are float64.
 template <class Q>
 __device__ __forceinline__ void clip_histogram(Q& q, uint32_t vmin, uint32_t vmax, double k, int maxiter, double* med_o,
                                                double* mean_o, double* sd_o)
@@ -198,21 +212,33 @@ __device__ __forceinline__ void clip_histogram(Q& q, uint32_t vmin, uint32_t vma
         m1 = (n & 1ull) ? m0 : q.select(lo.c + n / 2);
         if (it >= maxiter) break;
         // med -/+ k sigma, with sigma = sqrt(n S2 - S1^2) / n
-        const DF sd = df_div(df_sqrt(df_from(n * S2 - S1 * S1)), (float)n);
+        const unsigned long long num = n * S2 - S1 * S1;
+        const DF sd = df_div(df_sqrt(df_from(num)), (float)n);
         DF med;
         med.hi = 0.5f * ((float)m0 + (float)m1);    // exact
         med.lo = 0.f;
         const DF fl = df_step(med, -kf, sd), fh = df_step(med, kf, sd);
-        float ca = ceilf(fl.hi), cb = floorf(fh.hi);
-        if (ca == fl.hi && fl.lo > 0.f) ca += 1.f;
-        if (cb == fh.hi && fh.lo < 0.f) cb -= 1.f;
-        uint32_t na = ca <= (float)a ? a : (uint32_t)ca;
-        uint32_t nbv = cb >= (float)b ? b : (cb < 0.f ? 0u : (uint32_t)cb);
-        if (nbv < na) { na = a; nbv = a; }   // cannot happen for k > 0 (median lies inside)
+        const float tol = 0x1p-40f * fmaf(kf, sd.hi, med.hi);
+        const float dl = (fl.hi - rintf(fl.hi)) + fl.lo, dh = (fh.hi - rintf(fh.hi)) + fh.lo;
+        uint32_t na, nbv;
+        if (fabsf(dl) > tol && fabsf(dh) > tol) {
+            float ca = ceilf(fl.hi), cb = floorf(fh.hi);
+            if (ca == fl.hi && fl.lo > 0.f) ca += 1.f;
+            if (cb == fh.hi && fh.lo < 0.f) cb -= 1.f;
+            na = ca <= (float)a ? a : (uint32_t)ca;
+            nbv = cb >= (float)b ? b : (cb < 0.f ? 0u : (uint32_t)cb);
+        } else {
+            const uint2 r = clip_bounds_f64(m0, m1, num, n, k, a, b);
+            na = r.x;
+            nbv = r.y;
+        }
+        // At clip_k = 1 the bounds of a two-valued box lie on its values, and
+        // rounding can put both inside: nothing more is clipped then
+        if (nbv < na) break;
         HistSums nlo = q.prefix(na);
         HistSums nhi = q.prefix(nbv + 1u);
         unsigned long long nn = nhi.c - nlo.c;
-        if (nn == n || q.failed) break;    // the kept set did not change (or the query failed)
+        if (nn == n || nn == 0 || q.failed) break;   // the kept set did not change (or emptied), or the query failed
         a = na; b = nbv; lo = nlo; hi = nhi;
         n = nn; S1 = nhi.s1 - nlo.s1; S2 = nhi.s2 - nlo.s2;
     }
