@@ -322,7 +322,7 @@ __global__ void __launch_bounds__(GR_NT) k_growth(Image im, SplineTab sb, Spline
             if (gs.gain > 0.f && F > 0.0) V = fma(F, gs.inv_gain, V);
             const int64_t o = (int64_t)s * nr + lane;
             flux[o] = F;
-            ferr[o] = sqrt_pos(V);
+            ferr[o] = V > 0.0 ? sqrt(V) : 0.0;
             flags[o] = rfl;
         }
         __syncwarp();

@@ -204,7 +204,7 @@ __device__ __forceinline__ FitPart fit_merge(const FitPart& a, const FitPart& b)
     if (b.c == 0.0) return a;
     FitPart r;
     r.c = a.c + b.c;
-    const double dx = b.mx - a.mx, dy = b.my - a.my, f = b.c * recip_pos(r.c), g = a.c * f;
+    const double dx = b.mx - a.mx, dy = b.my - a.my, f = b.c / r.c, g = a.c * f;
     r.mx = fma(dx, f, a.mx);
     r.my = fma(dy, f, a.my);
     r.sxx = fma(dx * dx, g, a.sxx + b.sxx);
