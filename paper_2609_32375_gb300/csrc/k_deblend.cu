@@ -488,12 +488,15 @@ __device__ __forceinline__ void db_tree(const DeblendArgs& A, const Team T, cons
     }
 }
 
-// The rounds on a box in shared memory.  A pixel's state: 0 unassigned,
-// ST_CAND a candidate, else its rank, with ST_ODD or ST_EVEN added in the round
-// it was assigned in (by the round's parity) and taken off in the next: in a
-// round, ranks are read from pixels without that round's mark.  Within a round
-// an unassigned pixel can only become a candidate, so setting ST_CAND's bits
-// claims it.
+// The rounds on a box in shared memory.  A pixel's state, 16 bits of a word
+// that it shares with a neighbour: 0 unassigned, ST_CAND a candidate, else its
+// rank, with ST_ODD or ST_EVEN added in the round it was assigned in (by the
+// round's parity) and taken off in the next: in a round, ranks are read from
+// pixels without that round's mark.  Within a round an unassigned pixel can
+// only become a candidate, so setting ST_CAND's bits claims it.
+// While the rounds run, threads change and read the two states of a word at
+// once, so every change is an atomic of the word and every read a volatile
+// load of it: no access meets one of another size.
 constexpr unsigned ST_ODD = 0x4000u, ST_EVEN = 0x8000u, ST_CAND = 0xc000u, ST_RANK = 0x3fffu;
 
 __device__ __forceinline__ void db_rounds_shared(const DeblendArgs& A, DbCtaShared& S, const DbScratch& s, int w, int h,
@@ -514,6 +517,8 @@ __device__ __forceinline__ void db_rounds_shared(const DeblendArgs& A, DbCtaShar
         o[4] = r ? 1 : 0; o[5] = d && l ? w - 1 : 0; o[6] = d ? w : 0; o[7] = d && r ? w + 1 : 0;
     };
     unsigned* const words = reinterpret_cast<unsigned*>(state);
+    auto at = [](int q) { return 16 * (q & 1); };
+    auto load = [&](int q) { return *(const volatile unsigned*)(words + (q >> 1)) >> at(q) & 0xffffu; };
     int c = 0, round = 0, last = 0;          // last: pixels assigned in the round before, in list c - 1
     for (int i = A.nthresh - 1; i >= 0; --i) {
         const float tl = i > 0 ? S.tlev[i] : -INFINITY;    // nu > -inf: any pixel of the segment
@@ -523,9 +528,9 @@ __device__ __forceinline__ void db_rounds_shared(const DeblendArgs& A, DbCtaShar
             neighbours(q, o);
             bool any = false;
 #pragma unroll
-            for (int j = 0; j < 8; ++j) any = any || (o[j] && (state[q + o[j]] & ST_RANK) != 0);
+            for (int j = 0; j < 8; ++j) any = any || (o[j] && (load(q + o[j]) & ST_RANK) != 0);
             if (any) {
-                state[q] = ST_CAND;
+                atomicOr(words + (q >> 1), ST_CAND << at(q));
                 put(c, db_append(&S.ctr[c]), q);
             }
         }
@@ -536,18 +541,21 @@ __device__ __forceinline__ void db_rounds_shared(const DeblendArgs& A, DbCtaShar
             ++round;
             const unsigned now = round & 1 ? ST_ODD : ST_EVEN;
             if (t == 0) S.ctr[cp] = 0;       // (its length is in `last`; filled again in the next round)
-            for (int k = t; k < last; k += n) state[get(cp, k)] &= ST_RANK;
+            for (int k = t; k < last; k += n) {
+                const int q = get(cp, k);
+                atomicAnd(words + (q >> 1), ~(ST_CAND << at(q)));
+            }
             for (int k = t; k < nc; k += n) {
                 const int q = get(c, k);
                 int o[8];
                 unsigned st[8], best = ST_CAND;
                 neighbours(q, o);
 #pragma unroll
-                for (int j = 0; j < 8; ++j) st[j] = o[j] ? state[q + o[j]] : ST_CAND;
+                for (int j = 0; j < 8; ++j) st[j] = o[j] ? load(q + o[j]) : ST_CAND;
 #pragma unroll
                 for (int j = 0; j < 8; ++j)
                     if (st[j] != 0 && (st[j] & ST_CAND) != ST_CAND && !(st[j] & now)) best = min(best, st[j] & ST_RANK);
-                state[q] = (unsigned short)(best | now);
+                atomicXor(words + (q >> 1), (ST_CAND ^ (best | now)) << at(q));     // from ST_CAND
                 // claim the unassigned neighbours in the level set
                 float nu[8];
 #pragma unroll
@@ -555,7 +563,7 @@ __device__ __forceinline__ void db_rounds_shared(const DeblendArgs& A, DbCtaShar
                 unsigned old[8], won = 0;
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
-                    const int p = q + o[j], sh = 16 * (p & 1);
+                    const int p = q + o[j], sh = at(p);
                     old[j] = nu[j] > tl ? atomicOr(words + (p >> 1), ST_CAND << sh) >> sh & 0xffffu : 1u;
                 }
 #pragma unroll
