@@ -1796,9 +1796,15 @@ size_t mesh_all_smem(int Mx, int My)
     return mesh_lu_offset((int)ns) + 8 * nl * sizeof(float);
 }
 
+// Meshes for k_mesh_all, whose splines are solved in float32: up to
+// MESH_SMEM_NODES nodes, and no axis so long (some 2,800 nodes and more) that 32
+// bytes a node and 32 a node of the longer axis exceed 220 KB.  Those lines
+// take the float64 solves of the larger meshes, although k_mesh_all's own
+// 20 bytes a node would fit.
 bool mesh_fits_smem(int Mx, int My)
 {
-    return (size_t)Mx * My <= (size_t)MESH_SMEM_NODES && mesh_all_smem(Mx, My) <= 220 * 1024;
+    const size_t ns = (size_t)(Mx | 1) * My, nl = Mx > My ? Mx : My;
+    return (size_t)Mx * My <= (size_t)MESH_SMEM_NODES && (((ns * 32 + 15) & ~(size_t)15) + 32 * nl) <= 220 * 1024;
 }
 
 MeshArgs mesh_args(const double* bkg_raw, const double* rms_raw, const int* valid, Axis ax, Axis ay, int fsize,
