@@ -305,7 +305,10 @@ __global__ void __launch_bounds__(FIT_NT) k_ropt_fit(const FitPart* __restrict__
         fit[0] = NAN; fit[1] = NAN; fit[2] = v.c; fit[3] = 1.0;
         return;
     }
-    const double a = v.sxy / v.sxx;
+    // a calibrator of radius 0 (log10 r = -inf) leaves no line, whichever
+    // merge brought it in: some give an infinite slope where centred sums
+    // about the common mean are NaN
+    const double a = isfinite(v.mx) && isfinite(v.my) ? v.sxy / v.sxx : (double)NAN;
     fit[0] = a; fit[1] = v.my - a * v.mx; fit[2] = v.c; fit[3] = 0.0;
 }
 
