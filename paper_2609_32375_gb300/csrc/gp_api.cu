@@ -781,7 +781,7 @@ gp_status gp_optimal_radius(gp_ctx* ctx, const gp_image* img, const gp_bkg* bkg,
     w.start = cv.take<int>((size_t)ncx * ncy);
     w.fill = cv.take<int>((size_t)ncx * ncy);
     w.items = cv.take<int>(cat->capacity > 0 ? cat->capacity : 1);
-    w.parts = cv.take<double>(cat->capacity > 4 ? 2 * (size_t)cat->capacity : 8);   // >= 7 per 64 rows
+    w.parts = cv.take<double>((size_t)ropt_parts(cat->capacity) * ROPT_PART_DOUBLES);
     if (!cv.ok()) return oom(cv);
     mark_to(ctx, 2, GP_NSTAGES - 1, st);
     if (cat->capacity > 0) {

@@ -89,9 +89,15 @@ cudaError_t launch_deblend(const Image& im, const SplineTab& sb, const SplineTab
 // are given; scratch of the isolation grid from iso_grid()
 struct RoptWork {
     int *count, *start, *fill, *items;
-    double* parts;        // the fit's sums by CTA: 7 doubles each, at most a CTA per 64 rows, at most ROPT_PARTS
+    double* parts;        // the fit's sums by CTA: ropt_parts(rows) times ROPT_PART_DOUBLES
 };
-constexpr int ROPT_PARTS = 152 * 8, ROPT_PART_DOUBLES = 7;
+constexpr int ROPT_PART_DOUBLES = 7, ROPT_PART_ROWS = 64;
+// CTAs of the calibrator test: one per ROPT_PART_ROWS rows, at most eight per SM
+inline int ropt_parts(int rows)
+{
+    const int n = (int)(((int64_t)rows + ROPT_PART_ROWS - 1) / ROPT_PART_ROWS);
+    return n < 1 ? 1 : n < 152 * 8 ? n : 152 * 8;
+}
 void iso_grid(int W, int H, float d_iso, double* cs, int* ncx, int* ncy);
 cudaError_t launch_ropt(const Image& im, const SplineTab& sb, const SplineTab& sr, const float* taps, int kw, int kh,
                         const gp_catalog& cat, const double* flux, const double* ferr, const uint32_t* gflags,

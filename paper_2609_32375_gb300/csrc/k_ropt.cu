@@ -29,9 +29,6 @@
 
 namespace gp {
 
-
-static_assert(sizeof(double) * ROPT_PART_DOUBLES == 56, "FitPart");
-
 struct RoptTaps {
     int kw, kh;
     float t[KMAX];
@@ -196,6 +193,7 @@ __global__ void __launch_bounds__(256) k_iso_fill(const double* __restrict__ xs,
 struct FitPart {
     double c, mx, my, sxx, sxy, lo, hi;
 };
+static_assert(sizeof(FitPart) == ROPT_PART_DOUBLES * sizeof(double), "the workspace holds a part of this size per CTA");
 
 // two sets as one (the pairwise update of centred sums)
 __device__ __forceinline__ FitPart fit_merge(const FitPart& a, const FitPart& b)
@@ -230,7 +228,7 @@ __device__ __forceinline__ FitPart fit_warp(FitPart v)
     return v;
 }
 
-constexpr int CAL_NT = 64;
+constexpr int CAL_NT = ROPT_PART_ROWS;
 
 // The calibrator test (cheap conditions first, then the isolation: no other
 // centroid closer than d_iso), and each CTA's part of the fit: float64 sums of
@@ -384,7 +382,7 @@ cudaError_t launch_ropt(const Image& im, const SplineTab& sb, const SplineTab& s
     k_iso_count<<<grid, 256, 0, st>>>(cat.x, cat.y, cat.n, cap, cs, ncx, ncy, w.count);
     k_iso_scan<<<1, 1024, 0, st>>>(w.count, ncell, w.start, w.fill);
     k_iso_fill<<<grid, 256, 0, st>>>(cat.x, cat.y, cat.n, cap, cs, ncx, ncy, w.start, w.fill, w.items);
-    const int cal = std::max(1, std::min((cap + CAL_NT - 1) / CAL_NT, ROPT_PARTS));
+    const int cal = ropt_parts(cap);
     FitPart* parts = reinterpret_cast<FitPart*>(w.parts);
     k_iso_calib<<<cal, CAL_NT, 0, st>>>(cat.x, cat.y, cat.n, cap, cs, ncx, ncy, (double)d_iso, w.start, w.count, w.items,
                                         cat.flags, gflags, flux, ferr, nu, kopt, nr, (double)snr_min, R, calib, parts);
