@@ -45,7 +45,7 @@ constexpr int GR_NONE = 0x7f;              // u of an empty entry
 
 // the ring lists: u | v << 8 (bytes), ring after ring, and the ring of each 32
 struct GrowthList {
-    uint16_t uv[GR_LIST];
+    alignas(16) uint16_t uv[GR_LIST];      // (read by words)
     int8_t ring[GR_LIST / 32];
 };
 
