@@ -900,9 +900,12 @@ __global__ void __launch_bounds__(WB_NT, 1024 / WB_NT) k_boxstats_win(const BoxA
 // of a 1 MP frame at mesh 64 and 106 us for a masked 9 MP one, where a bitonic
 // sort of each box (78 block-wide steps of 4,096 values) took 183 and 721; the
 // quantiles of a 17 MP frame take 91 us against 523.  Two float32 values take one paired operation
-// in the compensated sums, and mean, sigma and range are float-float too, on
-// one warp: this GPU issues a float64 warp instruction every 16 cycles an SM,
-// and its long latency sits in the chain of every pass.
+// in the compensated sums.  The box's mean and sigma are float64; a pass takes
+// its mean to the 48 bits that the deviations can use, and its range in
+// float-float where that names the same values as float64 would, on one warp:
+// this GPU issues a float64 warp instruction every 16 cycles an SM, and its long
+// latency sits in the chain of every pass (float64 means there: 1 MP extraction
+// 140 -> 145 us, masked 9 MP 309 -> 319).
 constexpr int F32_LIST = 64;      // values among which the median is ranked
 
 template <int NT>
@@ -923,6 +926,21 @@ struct F32Box {
     uint32_t flag[SEL_BPT * NT / 32];     // a bit per bin: holds a quantile
 };
 
+// s / n to 48 bits (as a float64 quotient split into two floats), n < 2^15:
+// the residual of each partial quotient is exact or a rounding below those bits
+__device__ __forceinline__ DF df_mean(DF s, float n)
+{
+    const DF a = df_fast(s.hi, s.lo);
+    const float in = 1.f / n, q = a.hi * in;
+    DF r;
+    r.hi = fmaf(-q, n, a.hi);
+    r.lo = 0.f;
+    df_add(r, a.lo);
+    const float q1 = r.hi * in, q2 = (fmaf(-q1, n, r.hi) + r.lo) * in;
+    DF m = df_fast(q, q1);
+    m.lo += q2;
+    return m;
+}
 // sum over the first NW lanes (a power of two), in lane 0 .. NW - 1
 template <int NW>
 __device__ __forceinline__ DF df_sum_lanes(DF v)
@@ -1017,6 +1035,18 @@ __device__ __forceinline__ int range_shift(uint32_t klo, uint32_t khi, int lb)
 {
     const int bits = 32 - __clz(khi - klo);
     return bits > lb ? bits - lb : 0;
+}
+
+// the smallest float >= med - k sigma and the largest <= med + k sigma, in
+// float64, with sigma = sqrt(dev / n) (out of line: few passes need it)
+__device__ __noinline__ float2 clip_bounds_f32(float med0, float med1, DF dev, uint32_t n, double k)
+{
+    const double med = 0.5 * ((double)med0 + (double)med1), sd = sqrt(fmax(df_value(dev), 0.0) / (double)n);
+    const double lo = med - k * sd, hi = med + k * sd;
+    float2 b = make_float2((float)lo, (float)hi);
+    if ((double)b.x < lo) b.x = nextafterf(b.x, INFINITY);
+    if ((double)b.y > hi) b.y = nextafterf(b.y, -INFINITY);
+    return b;
 }
 
 template <int NT, int VPT, bool QUANT>
@@ -1179,7 +1209,9 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_boxstats_f32(const BoxArgs* _
 
     float flo = key_value(klo), fhi = key_value(khi);     // the kept range
     uint32_t n = 0, below = 0;                            // kept values; those dropped below the range
-    DF med = df_zero(), mean = df_zero(), sd = df_zero();   // (lane 0 of warp 0)
+    // of the kept set, in warp 0: sum, the two middle values, sum of squared deviations
+    DF sum = df_zero(), dev = df_zero();
+    float med0 = 0.f, med1 = 0.f;
     const float kf = (float)k;                            // clip_k is a float
     bool rebuild = false;
     for (int it = 0;; ++it) {
@@ -1221,8 +1253,8 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_boxstats_f32(const BoxArgs* _
         }
         const uint32_t r0 = below + (n - 1) / 2, r1 = below + n / 2;
         if (warp == 0) {
-            s = df_sum_lanes<NW>(S.red[lane < NW ? lane : 0]);
-            mean = df_div(df_fast(s.hi, s.lo), (float)n);
+            sum = df_sum_lanes<NW>(S.red[lane < NW ? lane : 0]);
+            const DF mean = df_mean(sum, (float)n);
             // the bins from the one with rank r0 to the one with rank r1 (those between are empty)
             const uint32_t b0 = find_bin<NT>(S, r0), b1 = r1 < S.pre[b0 + 1] ? b0 : find_bin<NT>(S, r1);
             if (lane == 0) {
@@ -1265,16 +1297,32 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_boxstats_f32(const BoxArgs* _
         if (!listed)                                      // many equal or close values
             k0 = block_select<NT>(each, key_of(blo), key_of(bhi), S.r, r1 > r0 ? &k1 : nullptr, S.sel);
         if (warp == 0) {
-            s = df_sum_lanes<NW>(S.red[lane < NW ? lane : 0]);
-            sd = df_sqrt(df_div(df_fast(s.hi, s.lo), (float)n));
+            dev = df_sum_lanes<NW>(S.red[lane < NW ? lane : 0]);
             if (listed) rank_list(S.list[0], S.nlist[0], S.r, S.r + (r1 - r0), &k0, &k1);
-            med = df_zero();
-            df_add(med, 0.5f * key_value(k0));
-            df_add(med, 0.5f * key_value(r1 == r0 ? k0 : k1));
+            med0 = key_value(k0);
+            med1 = key_value(r1 == r0 ? k0 : k1);
+            DF med = df_zero();
+            df_add(med, 0.5f * med0);
+            df_add(med, 0.5f * med1);
+            const DF sd = df_sqrt(df_div(df_fast(dev.hi, dev.lo), (float)n));
+            const DF lo = df_step(med, -kf, sd), hi = df_step(med, kf, sd);
+            // the float beyond each bound: its nearest float is lo.hi, lo.lo
+            // away.  Within 2^-40 of the terms float64 decides (an error of
+            // the float-float bound is below 2^-44 of them).
+            const float tol = 0x1p-40f * fmaf(kf, sd.hi, fabsf(med.hi));
+            float bl, bh;
+            if (fabsf(lo.lo) > tol && fabsf(hi.lo) > tol) {
+                bl = df_bound(lo, 1.f);
+                bh = df_bound(hi, -1.f);
+            } else {
+                const float2 b = clip_bounds_f32(med0, med1, dev, n, k);
+                bl = b.x;
+                bh = b.y;
+            }
             if (lane == 0) {
                 // values >= med - k sd and <= med + k sd
-                const float nlo = fmaxf(flo, df_bound(df_step(med, -kf, sd), 1.f));
-                const float nhi = fminf(fhi, df_bound(df_step(med, kf, sd), -1.f));
+                const float nlo = fmaxf(flo, bl);
+                const float nhi = fminf(fhi, bh);
                 S.flo = nlo;
                 S.fhi = nhi;
                 S.rebuild = nlo <= nhi && shift > 0 && (key_of(nhi) - key_of(nlo)) < (khi - klo) / 8;
@@ -1288,7 +1336,8 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_boxstats_f32(const BoxArgs* _
     }
     if (tid == 0) {
         double bb, rr;
-        box_result(df_value(med), df_value(mean), df_value(sd), &bb, &rr);
+        box_result(0.5 * ((double)med0 + (double)med1), df_value(sum) / (double)n,
+                   sqrt(fmax(df_value(dev), 0.0) / (double)n), &bb, &rr);
         A.bkg[box] = valid ? bb : 0.0;
         A.rms[box] = valid ? rr : 0.0;
         A.valid[box] = valid;
