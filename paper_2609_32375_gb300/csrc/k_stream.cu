@@ -12,10 +12,10 @@
 
 namespace gp {
 
-cudaError_t launch_stream_u16(const DetectArgs& one, const DetectArgs* batch, int nframes, int maxcta, int rows,
-                              bool fast, const CUtensorMap* maps, cudaStream_t st);
-cudaError_t launch_stream_f32(const DetectArgs& one, const DetectArgs* batch, int nframes, int maxcta, int rows,
-                              bool fast, const CUtensorMap* maps, cudaStream_t st);
+cudaError_t launch_stream_u16(const DetectArgs* args, const DetectArgs* batch, int nframes, bool fast,
+                              const CUtensorMap* maps, cudaStream_t st);
+cudaError_t launch_stream_f32(const DetectArgs* args, const DetectArgs* batch, int nframes, bool fast,
+                              const CUtensorMap* maps, cudaStream_t st);
 
 // ------------------------------------------------------- given masks ---
 // gp_label_mask: the caller's byte mask packed into the same bit layout,
@@ -122,26 +122,27 @@ int stream_ks(int kw, int kh)
     return k <= 3 ? 3 : k <= 5 ? 5 : k <= 7 ? 7 : 15;
 }
 
-static int stream_ctas(int W, int H, int rows)
+int stream_ctas(int W, int H, int rows)
 {
     return ((W + ST_COLS - 1) / ST_COLS) * ((H + rows - 1) / rows);
 }
 
 // Output rows per CTA.  A CTA takes about as long as its row groups, alone on
-// an SM or with three others there (the most that fit), so the pass lasts its
-// waves of 4 x 152 CTAs times the groups of one, and 1.5 more for filling the
-// pipeline.  Shorter CTAs read and filter more halo rows (8 groups of 5 for
-// 32 rows, 27 for 128).  1 MP float32: 85 us at 128 rows, 33 at 32; 4 MP
-// uint16: 75 and 32; 17 MP float32: 92 and 64 (64 rows).
-static int stream_rows(const DetectArgs* args, int n, int G)
+// an SM or with as many others as fit (four for 3 and 5 taps by tensor maps,
+// down to one for 15 taps of float32), so the pass lasts its waves of resident
+// x 152 CTAs times the groups of one, and 1.5 more for filling the pipeline.
+// Shorter CTAs read and filter more halo rows (8 groups of 5 for 32 rows, 27
+// for 128).  1 MP float32, 5 taps: 85 us at 128 rows, 33 at 32; 4 MP uint16: 75
+// and 32; 17 MP float32: 92 and 64 (64 rows).
+int stream_rows(const DetectArgs* args, int n, int G, int resident)
 {
     int best = ST_RC;
     double least = 0.0;
     for (int rows = ST_RC; rows >= TY; rows >>= 1) {
         int64_t ctas = 0;
         for (int f = 0; f < n; ++f) ctas += stream_ctas(args[f].im.W, args[f].im.H, rows);
-        const int groups = (rows + 2 * (args[0].ks / 2) + G - 1) / G;
-        const double t = (double)((ctas + 4 * 152 - 1) / (4 * 152)) * (groups + 1.5);
+        const int groups = (rows + 2 * (args[0].ks / 2) + G - 1) / G, wave = resident * 152;
+        const double t = (double)((ctas + wave - 1) / wave) * (groups + 1.5);
         if (rows == ST_RC || t < least) {
             least = t;
             best = rows;
@@ -161,19 +162,17 @@ cudaError_t launch_stream_any(const DetectArgs* args, const DetectArgs* batch, i
         else k_pack_mask<false><<<blocks, 128, 0, st>>>(nullptr, one);
         return cudaGetLastError();
     }
-    const int G = stream_group_rows(one.ks), rows = stream_rows(args, nframes, G);
+    const int G = stream_group_rows(one.ks);
     CUtensorMap maps[MAX_BATCH];
     bool fast = one.nrank == 1 && one.ks <= 7, tma = true;
-    int ctas = 0;
     for (int f = 0; f < nframes; ++f) {
         const DetectArgs& A = args[f];
         fast = fast && !A.mask_out && !A.nnear && !A.im.mask;
         tma = tma && make_tmap(A.im, G, maps + f);
-        ctas = std::max(ctas, stream_ctas(A.im.W, A.im.H, rows));
     }
     const CUtensorMap* mp = tma ? maps : nullptr;
-    if (one.im.is_f32) return launch_stream_f32(one, batch, nframes, ctas, rows, fast, mp, st);
-    return launch_stream_u16(one, batch, nframes, ctas, rows, fast, mp, st);
+    if (one.im.is_f32) return launch_stream_f32(args, batch, nframes, fast, mp, st);
+    return launch_stream_u16(args, batch, nframes, fast, mp, st);
 }
 
 }  // namespace gp

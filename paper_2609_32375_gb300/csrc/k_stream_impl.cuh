@@ -45,7 +45,8 @@
 // A CTA's rows (a multiple of TY, at most ST_RC) are chosen by the launcher:
 // a group takes about 3 us whatever else the SM runs (a chain of dependent
 // steps within each warp), so a frame that does not fill the SMs with
-// 128-row CTAs is cut into shorter ones (stream_rows).
+// 128-row CTAs is cut into shorter ones (stream_rows), by the number of CTAs
+// of the instance that an SM holds.
 // The ring keeps two groups.  The filter pass reads other lanes' columns only
 // in the current group's rows (a warp writes the next group's rows after the
 // barrier that ends every warp's pass over them); the previous group's rows
@@ -345,8 +346,18 @@ constexpr int stream_nmaps(int mode) { return mode == SM_BATCH_TMA ? MAX_BATCH :
 // FAST: one separable term, no input mask, neither the byte mask nor the
 // near-threshold count requested -- the form the pipeline runs on the
 // workloads; the general form handles the rest.
+// CTAs an SM holds at least (0: no bound).  7 taps of uint16 by tensor maps come out at 130 to
+// 136 registers, two above what four CTAs allow (a 36 MP frame then takes two
+// waves, 186 us for 116); the float32 form is held to two by its stages, and the
+// others need no bound or would spill.
+template <bool F32, int KS, int MODE>
+constexpr int stream_min_ctas()
+{
+    return !F32 && KS == 7 && (MODE == SM_TMA || MODE == SM_BATCH_TMA) ? 4 : 0;
+}
+
 template <bool F32, int KS, int MODE, bool FAST>
-__global__ void __launch_bounds__(ST_NT) k_stream(const DetectArgs* __restrict__ batch,
+__global__ void __launch_bounds__(ST_NT, stream_min_ctas<F32, KS, MODE>()) k_stream(const DetectArgs* __restrict__ batch,
                                                   const __grid_constant__ DetectArgs one, int rows,
                                                   const __grid_constant__ StreamMaps<stream_nmaps(MODE)> maps)
 {
@@ -740,56 +751,74 @@ __global__ void __launch_bounds__(ST_NT) k_stream(const DetectArgs* __restrict__
     }
 }
 
+// k_stream.cu: output rows per CTA of n frames, for an instance of G-row
+// groups of which an SM holds `resident` CTAs; the CTAs of a frame
+int stream_rows(const DetectArgs* args, int n, int G, int resident);
+int stream_ctas(int W, int H, int rows);
+
 template <bool F32, int KS, int MODE, bool FAST>
-cudaError_t launch_stream_inst(const DetectArgs& one, const DetectArgs* batch, int nframes, int maxcta, int rows,
-                               const CUtensorMap* maps, cudaStream_t st)
+cudaError_t launch_stream_inst(const DetectArgs* args, const DetectArgs* batch, int nframes, const CUtensorMap* maps,
+                               cudaStream_t st)
 {
     const size_t smem = StreamSmem<KS>::total(F32 ? 4 : 2);
     auto* fn = k_stream<F32, KS, MODE, FAST>;
-    cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    // a property of the compiled kernel
+    static const int resident = [&] {
+        int n = 0;
+        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn, ST_NT, smem) == cudaSuccess && n > 0 ? n : 1;
+    }();
+    const int rows = stream_rows(args, nframes, StreamCfg<KS>::G, resident);
+    int ctas = 0;
+    for (int f = 0; f < nframes; ++f) {
+        const int c = stream_ctas(args[f].im.W, args[f].im.H, rows);
+        ctas = c > ctas ? c : ctas;
+    }
     StreamMaps<stream_nmaps(MODE)> m;
     memset(&m, 0, sizeof m);
     if (maps) memcpy(m.m, maps, sizeof(CUtensorMap) * (MODE == SM_BATCH_TMA ? nframes : 1));
-    launch_dep(fn, dim3(maxcta, nframes), dim3(ST_NT), smem, st, batch, one, rows, m);
+    launch_dep(fn, dim3(ctas, nframes), dim3(ST_NT), smem, st, batch, args[0], rows, m);
     return cudaGetLastError();
 }
 
 // the instances of one dtype (k_stream_u16.cu, k_stream_f32.cu); maps: a
 // tensor map per frame, or null (DIRECT staging)
 template <bool F32>
-cudaError_t launch_stream_dtype(const DetectArgs& one, const DetectArgs* batch, int nframes, int maxcta, int rows,
-                                bool fast, const CUtensorMap* maps, cudaStream_t st)
+cudaError_t launch_stream_dtype(const DetectArgs* args, const DetectArgs* batch, int nframes, bool fast,
+                                const CUtensorMap* maps, cudaStream_t st)
 {
+    const int ks = args[0].ks;
     if (batch) {
         // FAST batches exist in the TMA form only; the rest take the general direct form
         if (maps && fast) {
-            switch (one.ks) {
-            case 3: return launch_stream_inst<F32, 3, SM_BATCH_TMA, true>(one, batch, nframes, maxcta, rows, maps, st);
-            case 5: return launch_stream_inst<F32, 5, SM_BATCH_TMA, true>(one, batch, nframes, maxcta, rows, maps, st);
-            case 7: return launch_stream_inst<F32, 7, SM_BATCH_TMA, true>(one, batch, nframes, maxcta, rows, maps, st);
+            switch (ks) {
+            case 3: return launch_stream_inst<F32, 3, SM_BATCH_TMA, true>(args, batch, nframes, maps, st);
+            case 5: return launch_stream_inst<F32, 5, SM_BATCH_TMA, true>(args, batch, nframes, maps, st);
+            case 7: return launch_stream_inst<F32, 7, SM_BATCH_TMA, true>(args, batch, nframes, maps, st);
             default: break;
             }
         }
-        switch (one.ks) {
-        case 3: return launch_stream_inst<F32, 3, SM_BATCH, false>(one, batch, nframes, maxcta, rows, nullptr, st);
-        case 5: return launch_stream_inst<F32, 5, SM_BATCH, false>(one, batch, nframes, maxcta, rows, nullptr, st);
-        case 7: return launch_stream_inst<F32, 7, SM_BATCH, false>(one, batch, nframes, maxcta, rows, nullptr, st);
-        default: return launch_stream_inst<F32, 15, SM_BATCH, false>(one, batch, nframes, maxcta, rows, nullptr, st);
+        switch (ks) {
+        case 3: return launch_stream_inst<F32, 3, SM_BATCH, false>(args, batch, nframes, nullptr, st);
+        case 5: return launch_stream_inst<F32, 5, SM_BATCH, false>(args, batch, nframes, nullptr, st);
+        case 7: return launch_stream_inst<F32, 7, SM_BATCH, false>(args, batch, nframes, nullptr, st);
+        default: return launch_stream_inst<F32, 15, SM_BATCH, false>(args, batch, nframes, nullptr, st);
         }
     }
-#define GP_STREAM_CASE(KSV)                                                                                       \
-    case KSV:                                                                                                     \
-        if (maps) return fast ? launch_stream_inst<F32, KSV, SM_TMA, true>(one, nullptr, 1, maxcta, rows, maps, st)  \
-                              : launch_stream_inst<F32, KSV, SM_TMA, false>(one, nullptr, 1, maxcta, rows, maps, st); \
-        return fast ? launch_stream_inst<F32, KSV, SM_DIRECT, true>(one, nullptr, 1, maxcta, rows, nullptr, st)      \
-                    : launch_stream_inst<F32, KSV, SM_DIRECT, false>(one, nullptr, 1, maxcta, rows, nullptr, st);
-    switch (one.ks) {
+#define GP_STREAM_CASE(KSV)                                                                          \
+    case KSV:                                                                                        \
+        if (maps) return fast ? launch_stream_inst<F32, KSV, SM_TMA, true>(args, nullptr, 1, maps, st)  \
+                              : launch_stream_inst<F32, KSV, SM_TMA, false>(args, nullptr, 1, maps, st); \
+        return fast ? launch_stream_inst<F32, KSV, SM_DIRECT, true>(args, nullptr, 1, nullptr, st)      \
+                    : launch_stream_inst<F32, KSV, SM_DIRECT, false>(args, nullptr, 1, nullptr, st);
+    switch (ks) {
         GP_STREAM_CASE(3)
         GP_STREAM_CASE(5)
         GP_STREAM_CASE(7)
     default:
-        if (maps) return launch_stream_inst<F32, 15, SM_TMA, false>(one, nullptr, 1, maxcta, rows, maps, st);
-        return launch_stream_inst<F32, 15, SM_DIRECT, false>(one, nullptr, 1, maxcta, rows, nullptr, st);
+        if (maps) return launch_stream_inst<F32, 15, SM_TMA, false>(args, nullptr, 1, maps, st);
+        return launch_stream_inst<F32, 15, SM_DIRECT, false>(args, nullptr, 1, nullptr, st);
     }
 #undef GP_STREAM_CASE
 }

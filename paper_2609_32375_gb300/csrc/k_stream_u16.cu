@@ -5,10 +5,10 @@
 
 namespace gp {
 
-cudaError_t launch_stream_u16(const DetectArgs& one, const DetectArgs* batch, int nframes, int maxcta, int rows,
-                             bool fast, const CUtensorMap* maps, cudaStream_t st)
+cudaError_t launch_stream_u16(const DetectArgs* args, const DetectArgs* batch, int nframes, bool fast,
+                             const CUtensorMap* maps, cudaStream_t st)
 {
-    return launch_stream_dtype<false>(one, batch, nframes, maxcta, rows, fast, maps, st);
+    return launch_stream_dtype<false>(args, batch, nframes, fast, maps, st);
 }
 
 }  // namespace gp
