@@ -18,10 +18,11 @@
 //    first pixels); the objects are labelled 1 + their minimum linear index.
 //
 // A team of threads per candidate segment, its bounding box in global
-// scratch: a warp for boxes up to DB_SMALL pixels, a CTA above, a cluster of 8
-// CTAs above DB_BIG.  One launch serves all three: its clusters first work
-// through the big candidates together, then each CTA through the middle ones,
-// then each warp through the small ones, all by claims on shared counters.
+// scratch: a warp for boxes up to DB_SMALL pixels, a group of DB_GW warps up to
+// DB_MED, a CTA above, a cluster of 8 CTAs above DB_BIG.  One launch serves all:
+// its clusters first work through the big candidates together, then each CTA
+// through the larger ones, each group through the middle ones and each warp
+// through the small ones, all by claims on shared counters.
 // The time is the largest candidate's: a nebulosity whose box holds 55,000
 // pixels takes 30 levels of five passes over its pixels, then some 250 growth
 // rounds, 0.96 ms in all (a single CTA took 6 to 15 ms on such a field).  The
@@ -50,13 +51,26 @@ namespace cg = cooperative_groups;
 
 constexpr int DB_NT = 1024;                   // one CTA an SM
 constexpr int DB_CL = 8;                     // CTAs of a cluster
-constexpr int DB_SMALL = 1024, DB_BIG = 8192;   // box pixels: a warp's most; a CTA's most
+// Box pixels: a warp's most, a group's most, a CTA's most.  The lone candidate
+// of a sparse frame sets the time there, so a team is as large as its box can
+// use: a warp takes 1.1 ms for a box of 1,000 pixels, a group 0.4, and the stars
+// of a 300 x 257 frame 0.43 ms in groups above 128 pixels, 0.74 above 256.  A 4 MP
+// CCD frame's 2,471 candidates take 0.60 ms with a warp's limit at 64 or 128
+// pixels, 0.74 at 256, 1.66 at 1,024 and no groups; groups of 4 warps 0.72; CTAs
+// in place of the groups 0.59, but then a crowded 17 MP field, whose groups
+// number thousands, 5 % more.  64 against 128: the 162 stars of a 512 x 512 frame
+// with boxes up to 100 pixels 0.30 and 0.38 ms.
+constexpr int DB_SMALL = 64, DB_MED = 1024, DB_BIG = 8192;
+constexpr int DB_GW = 8;                     // warps of a group
 constexpr int DB_ROW = 1024;                 // box pixels of an object's catalog row: a warp's most
 // the call's counters, one 256-byte block cleared per call: candidates larger
 // than DB_SMALL, staged objects, small candidates, big ones; the next big,
-// middle and small one to claim; then the first big candidates' indexes (any
-// more count as middle ones)
-enum { DBC_N = 0, DBC_OBJ = 1, DBC_SMALL = 2, DBC_BIG = 3, DBC_NEXT_BIG = 4, DBC_NEXT = 5, DBC_NEXT_SMALL = 6, DBC_LIST = 8 };
+// CTA's, small and group's one to claim; then the first big candidates' indexes
+// (any more are a CTA's)
+enum {
+    DBC_N = 0, DBC_OBJ = 1, DBC_SMALL = 2, DBC_BIG = 3, DBC_NEXT_BIG = 4, DBC_NEXT = 5, DBC_NEXT_SMALL = 6, DBC_NEXT_MED = 7,
+    DBC_LIST = 8
+};
 constexpr int DB_CTL = 64, DB_MAX_BIG = DB_CTL - DBC_LIST;
 constexpr int DB_MAX_SEEDS = 1024;
 constexpr int DB_MAX_LEVELS = 64;            // nthresh at most (checked by the API)
@@ -77,8 +91,8 @@ struct DeblendArgs {
     const uint32_t* label;
     const int* npix;
     const int *xmin, *xmax, *ymin, *ymax;
-    // candidates (the larger ones from the front, the small ones from the
-    // back), counters and scratch
+    // candidates (the larger ones from the front, a group's as ~row; the small
+    // ones from the back), counters and scratch
     int* cand;
     int* ctl;
     int64_t* off;            // [cand] first scratch byte of each candidate (-1: no room)
@@ -192,9 +206,10 @@ struct DbWarpShared {
     float tlev[DB_MAX_LEVELS + 1];
 };
 
+// WIDE: a CTA or more, with the shared memory of one
 struct WarpTeam {
     using Inner = WarpTeam;
-    static constexpr bool CLUSTER = false;
+    static constexpr bool CLUSTER = false, WIDE = false;
     __device__ bool leads() const { return true; }
     __device__ Inner inner() const { return *this; }
     int* ctr;
@@ -206,6 +221,47 @@ struct WarpTeam {
     __device__ long long sum(long long v) const { return warp_sum64(v); }
     __device__ int max(int v) const { return __reduce_max_sync(0xffffffffu, v); }
 };
+
+struct DbGroupShared {
+    int ctr[4];
+    float tlev[DB_MAX_LEVELS + 1];
+    long long part[DB_GW];
+    int next;
+};
+
+// DB_GW warps of a CTA, on a named barrier of their own
+struct GroupTeam {
+    using Inner = GroupTeam;
+    static constexpr bool CLUSTER = false, WIDE = false;
+    DbGroupShared& s;
+    int* ctr;
+    float* tlev;
+    __device__ GroupTeam(DbGroupShared& sh) : s(sh), ctr(sh.ctr), tlev(sh.tlev) {}
+    __device__ bool leads() const { return true; }
+    __device__ Inner inner() const { return *this; }
+    __device__ int t() const { return threadIdx.x % (32 * DB_GW); }
+    __device__ int n() const { return 32 * DB_GW; }
+    __device__ void sync() const
+    {
+        asm volatile("barrier.sync %0, %1;" ::"r"(1 + (int)threadIdx.x / (32 * DB_GW)), "n"(32 * DB_GW) : "memory");
+    }
+    template <class Op>
+    __device__ long long all(long long v, Op op) const
+    {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v = op(v, __shfl_xor_sync(0xffffffffu, v, o));
+        if ((threadIdx.x & 31) == 0) s.part[t() >> 5] = v;
+        sync();
+        v = s.part[0];
+#pragma unroll
+        for (int w = 1; w < DB_GW; ++w) v = op(v, s.part[w]);
+        sync();
+        return v;
+    }
+    __device__ long long sum(long long v) const { return all(v, [](long long a, long long b) { return a + b; }); }
+    __device__ int max(int v) const { return (int)all(v, [](long long a, long long b) { return a > b ? a : b; }); }
+};
+static_assert(DB_NT % (32 * DB_GW) == 0 && DB_NT / (32 * DB_GW) < 16, "groups of whole warps, a named barrier each");
 
 constexpr int DB_LIST = 1024;                // candidates of a round in shared memory; more go to global
 struct DbCtaShared {
@@ -225,7 +281,7 @@ constexpr size_t DB_SMEM = 2 * (size_t)DB_BOX;
 template <int CL>
 struct CtaTeam {
     using Inner = CtaTeam<1>;
-    static constexpr bool CLUSTER = CL > 1;
+    static constexpr bool CLUSTER = CL > 1, WIDE = true;
     __device__ bool leads() const { return rank() == 0; }
     __device__ Inner inner() const { return Inner(s); }
     __device__ DbCtaShared& first() const
@@ -607,7 +663,7 @@ template <class Team>
 __device__ __forceinline__ void db_growth(const DeblendArgs& A, const Team T, const DbScratch& s, int w, int h, int Ar)
 {
     extern __shared__ __align__(16) unsigned char box[];
-    constexpr bool BUCKETS = !std::is_same<Team, WarpTeam>::value;
+    constexpr bool BUCKETS = Team::WIDE;
     int* cur = s.own;
     int* stamp = s.own2;
     if constexpr (BUCKETS) {
@@ -745,7 +801,7 @@ __device__ __noinline__ void db_segment(const DeblendArgs& A, int ci, const Team
     const int W = im.W, H = im.H;
     const int hx = A.kw / 2, hy = A.kh / 2;
     if (A.off[ci] < 0) return;                         // no room: left as it is (status set)
-    const int r = A.cand[ci];
+    const int rc = A.cand[ci], r = rc < 0 ? ~rc : rc;
     const uint32_t L = A.label[r];
     const int x0 = A.xmin[r], x1 = A.xmax[r], y0 = A.ymin[r], y1 = A.ymax[r];
     const int w = x1 - x0 + 1, h = y1 - y0 + 1, Ar = w * h;
@@ -926,11 +982,11 @@ __device__ __noinline__ void db_segment(const DeblendArgs& A, int ci, const Team
     const int lane = threadIdx.x & 31, gw = t >> 5, nw = n >> 5;
     for (int k = gw; k < ns; k += nw) {
         const int bw = bx1[k] - bx0[k] + 1, area = bw * (by1[k] - by0[k] + 1);
-        if (nw > 1 && area > DB_ROW) continue;
+        if (Team::WIDE && area > DB_ROW) continue;
         const DbSums v = db_object_sums<F32>(im, s, cur, k + 1, x0, y0, w, wh, hx, hy, bx0[k], by0[k], bw, area, lane, 32);
         if (lane == 0) db_emit(A, v, L, label(k), x0, y0, w, bx0[k], bx1[k], by0[k], by1[k]);
     }
-    if constexpr (!std::is_same<Team, WarpTeam>::value) {
+    if constexpr (Team::WIDE) {
         static_assert(sizeof(T.s.list) >= sizeof(long long) * DB_SUM_WORDS * (DB_NT / 32), "the warps' sums fit");
         long long* part = reinterpret_cast<long long*>(T.s.list);
         int large = 0;
@@ -969,10 +1025,18 @@ __device__ __noinline__ void db_segment(const DeblendArgs& A, int ci, const Team
 template <bool F32>
 __global__ void __cluster_dims__(DB_CL, 1, 1) __launch_bounds__(DB_NT, 1) k_deblend(const __grid_constant__ DeblendArgs A)
 {
+    const int nbig = min(A.ctl[DBC_BIG], DB_MAX_BIG), nmid = A.ctl[DBC_N], nsmall = A.ctl[DBC_SMALL];
     __shared__ DbCtaShared sh;
+    __shared__ DbGroupShared gs[DB_NT / (32 * DB_GW)];
     __shared__ DbWarpShared ws[DB_NT / 32];
     __shared__ int next;
-    const int nbig = min(A.ctl[DBC_BIG], DB_MAX_BIG), nmid = A.ctl[DBC_N], nsmall = A.ctl[DBC_SMALL];
+    // the next candidate of the front that is (not) a group's
+    auto claim = [&](int* counter, bool group) {
+        int c;
+        do c = atomicAdd(counter, 1);
+        while (c < nmid && (A.cand[c] < 0) != group);
+        return c;
+    };
     {
         const CtaTeam<DB_CL> T(sh);
         const auto cl = cg::this_cluster();
@@ -989,13 +1053,25 @@ __global__ void __cluster_dims__(DB_CL, 1, 1) __launch_bounds__(DB_NT, 1) k_debl
     for (;;) {
         const CtaTeam<1> T(sh);
         __syncthreads();
-        if (threadIdx.x == 0) next = atomicAdd(A.ctl + DBC_NEXT, 1);
+        if (threadIdx.x == 0) next = claim(A.ctl + DBC_NEXT, false);
         __syncthreads();
         const int c = next;
         if (c >= nmid) break;
         bool big = false;
         for (int b = 0; b < nbig; ++b) big = big || A.ctl[DBC_LIST + b] == c;
         if (!big) db_segment<F32>(A, c, T);
+    }
+    {
+        DbGroupShared& g = gs[threadIdx.x / (32 * DB_GW)];
+        const GroupTeam T(g);
+        for (;;) {
+            T.sync();
+            if (T.t() == 0) g.next = claim(A.ctl + DBC_NEXT_MED, true);
+            T.sync();
+            const int c = g.next;
+            if (c >= nmid) break;
+            db_segment<F32>(A, c, T);
+        }
     }
     const WarpTeam T(ws[threadIdx.x >> 5]);
     for (;;) {
@@ -1009,7 +1085,8 @@ __global__ void __cluster_dims__(DB_CL, 1, 1) __launch_bounds__(DB_NT, 1) k_debl
 }
 
 // candidates: rows with at least 2 minarea pixels, their scratch bytes; the
-// larger ones from the front of the arrays, the small ones from the back
+// larger ones from the front of the arrays (a group's as ~row), the small ones
+// from the back
 __global__ void __launch_bounds__(256) k_db_select(const int* __restrict__ n_dev, int cap,
                                                    const int* __restrict__ npix, const int* __restrict__ xmin,
                                                    const int* __restrict__ xmax, const int* __restrict__ ymin,
@@ -1027,7 +1104,7 @@ __global__ void __launch_bounds__(256) k_db_select(const int* __restrict__ n_dev
             const int b = atomicAdd(ctl + DBC_BIG, 1);
             if (b < DB_MAX_BIG) ctl[DBC_LIST + b] = k;
         }
-        cand[k] = r;
+        cand[k] = !small && w * h <= DB_MED ? ~r : r;
         bytes[k] = db_scratch_bytes(w * h, (w + 2 * hx) * (h + 2 * hy));
     }
 }
