@@ -346,14 +346,16 @@ constexpr int stream_nmaps(int mode) { return mode == SM_BATCH_TMA ? MAX_BATCH :
 // FAST: one separable term, no input mask, neither the byte mask nor the
 // near-threshold count requested -- the form the pipeline runs on the
 // workloads; the general form handles the rest.
-// CTAs an SM holds at least (0: no bound).  7 taps of uint16 by tensor maps come out at 130 to
-// 136 registers, two above what four CTAs allow (a 36 MP frame then takes two
-// waves, 186 us for 116); the float32 form is held to two by its stages, and the
-// others need no bound or would spill.
+// CTAs an SM holds at least (0: no bound), for uint16 by tensor maps.  7 taps
+// come out at 130 to 136 registers, two above what four CTAs allow: a 36 MP
+// frame then takes two waves, 186 us for 121.  3 taps come out at 96, as if for
+// a fifth CTA that the shared memory does not hold: 119 us for 105.  The float32
+// form of 7 taps is held to two by its stages, and the others need no bound or
+// would spill.
 template <bool F32, int KS, int MODE>
 constexpr int stream_min_ctas()
 {
-    return !F32 && KS == 7 && (MODE == SM_TMA || MODE == SM_BATCH_TMA) ? 4 : 0;
+    return !F32 && (KS == 3 || KS == 7) && (MODE == SM_TMA || MODE == SM_BATCH_TMA) ? 4 : 0;
 }
 
 template <bool F32, int KS, int MODE, bool FAST>
