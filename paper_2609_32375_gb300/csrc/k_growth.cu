@@ -349,8 +349,9 @@ cudaError_t launch_growth(const Image& im, const SplineTab& sb, const SplineTab&
     gs.gain = gain;
     gs.inv_gain = gain > 0.f ? 1.0 / (double)gain : 0.0;
     GrowthList gl;
-    if (gs.rmax <= 40) {
-        int cnt[GP_GROWTH_MAX_NR] = {}, at[GP_GROWTH_MAX_NR], ring[40 * 40 + 1], total = 0;
+    constexpr int RMAX_LIST = 36;            // a disc of radius 37 alone has more than GR_LIST pixels
+    if (gs.rmax <= RMAX_LIST) {
+        int cnt[GP_GROWTH_MAX_NR] = {}, at[GP_GROWTH_MAX_NR], ring[RMAX_LIST * RMAX_LIST + 1], total = 0;
         for (int d2 = 0, k = 0; d2 <= gs.rmax * gs.rmax; ++d2) {
             while (gs.r[k] * gs.r[k] < d2) ++k;
             ring[d2] = k;
