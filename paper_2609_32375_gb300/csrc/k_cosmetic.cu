@@ -19,7 +19,7 @@
 // Both filters change few pixels, so both first ask a cheap question whose
 // "no" is certain, and take the medians only where the answer is "maybe":
 //   k_rtn  the 3 x 3 median lies between the smallest and the largest of the
-//          window's three row medians;
+//          window's three row medians (small frames: every median, by blocks);
 //   k_cr   med5(I) is at least the smallest of the window's five column
 //          medians (15 of the 25 values are no less), which bounds S from
 //          above before its own median is taken off (that is never negative).
@@ -453,7 +453,7 @@ __device__ __forceinline__ float med3_nan(float a, float b, float c)
     return max_nan(min_nan(a, b), min_nan(max_nan(a, b), c));
 }
 
-// A warp takes 128 columns, a lane 4 of them, over RTN_ROWS rows, with the
+// A warp takes 128 columns, a lane 4 of them, over ROWS rows, with the
 // medians of 3 along three rows in registers; neighbours' columns come by
 // shuffle.  The window's median lies between the smallest and the largest of
 // its three row medians (6 of the 9 values are no less than the smallest), so
@@ -462,11 +462,13 @@ __device__ __forceinline__ float med3_nan(float a, float b, float c)
 // registers; an outlier's 8 neighbours are then tested by 8 lanes, or by its
 // own lane where a row holds many (a track).  Bound by the row loop's latency.  17 MP after the cosmic-ray filter: 153 us with the median
 // taken at every pixel of 32 x 32 blocks in shared memory, 87 us so.
-constexpr int RTN_ROWS = 8;
 constexpr int RTN_NT = 64;
-constexpr int RTN_FEW = 6;      // lanes with outliers in a row: up to this many, a warp for each
+// lanes with outliers in a row: up to this many, the warp's lanes test one's
+// neighbours together, a round trip each; more (a track along the row) and each
+// lane tests its own, eight round trips at most for all
+constexpr int RTN_FEW = 6;
 
-template <bool F32>
+template <bool F32, int ROWS>
 __global__ void __launch_bounds__(RTN_NT) k_rtn(const __grid_constant__ RtnArgs A, bool vec, bool ovec)
 {
     using T = typename std::conditional<F32, float, uint16_t>::type;
@@ -474,9 +476,9 @@ __global__ void __launch_bounds__(RTN_NT) k_rtn(const __grid_constant__ RtnArgs 
     const int W = im.W, H = im.H;
     const int lane = threadIdx.x & 31, nx = (W + 127) / 128;
     const int wid = blockIdx.x * (RTN_NT / 32) + (threadIdx.x >> 5);
-    const int y0 = wid / nx * RTN_ROWS, x0 = (wid % nx) * 128 + 4 * lane;
+    const int y0 = wid / nx * ROWS, x0 = (wid % nx) * 128 + 4 * lane;
     if (y0 >= H) return;
-    const int y1 = min(y0 + RTN_ROWS, H);
+    const int y1 = min(y0 + ROWS, H);
     // the lane's columns in the frame (mirrored beyond it), and the ones
     // beside the warp's that lanes 0 and 31 fetch
     int mx[4];
@@ -647,6 +649,67 @@ __global__ void __launch_bounds__(RTN_NT) k_rtn(const __grid_constant__ RtnArgs 
     if (lane == 0 && A.count && nrep) atomicAdd(A.count, nrep);
 }
 
+// Small frames: 32 x 32 blocks in shared memory, the median of every pixel.
+// No step of it waits for a row's outliers, which set k_rtn's time where the
+// chip is not filled.  CLEAN: the frame cannot hold a bad pixel (uint16 without a
+// mask); else each CTA looks whether its part does.
+template <bool F32, bool CLEAN>
+__global__ void __launch_bounds__(CM_NT) k_rtn_block(const __grid_constant__ RtnArgs A)
+{
+    constexpr int HA = 2, NA = CM_B + 2 * HA;
+    constexpr int HO = 1, NO = CM_B + 2 * HO;
+    __shared__ float a[NA][NA];
+    __shared__ float med[NO][NO];
+    __shared__ uint8_t outl[NO][NO];
+    __shared__ int nrep;
+    const Image& im = A.im;
+    const int W = im.W, H = im.H;
+    const int X0 = blockIdx.x * CM_B, Y0 = blockIdx.y * CM_B;
+    const int t = threadIdx.x;
+    if (t == 0) nrep = 0;
+    bool odd = false;
+    for (int p = t; p < NA * NA; p += CM_NT) {
+        const int r = p / NA, c = p - r * NA;
+        const float v = pixel_or_nan<F32>(im, mirror_idx(X0 - HA + c, W), mirror_idx(Y0 - HA + r, H));
+        a[r][c] = v;
+        if (!CLEAN) odd = odd || isnan(v);
+    }
+    if constexpr (CLEAN) __syncthreads();
+    else odd = __syncthreads_or(odd);
+    for (int p = t; p < NO * NO; p += CM_NT) {
+        const int r = p / NO, c = p - r * NO;
+        float v[9];
+#pragma unroll
+        for (int k = 0; k < 9; ++k) v[k] = a[r + k / 3][c + k % 3];
+        float m;
+        if (!CLEAN && odd) m = median_net<9, 16>(v);
+        else m = med_sel<9>(v);
+        const float x = a[r + 1][c + 1];
+        med[r][c] = m;
+        outl[r][c] = (!isnan(x) && fabsf(x - m) > A.t) ? 1 : 0;      // NaN comparisons are false
+    }
+    __syncthreads();
+    for (int p = t; p < CM_B * CM_B; p += CM_NT) {
+        const int r = p / CM_B, c = p - r * CM_B;
+        const int x = X0 + c, y = Y0 + r;
+        if (x >= W || y >= H) continue;
+        bool rep = outl[r + 1][c + 1];
+        for (int dy = 0; dy < 3 && rep; ++dy)
+            for (int dx = 0; dx < 3; ++dx)
+                if ((dy != 1 || dx != 1) && outl[r + dy][c + dx]) { rep = false; break; }
+        bool unused;
+        const int64_t i = (int64_t)y * W + x;
+        A.out[i] = rep ? med[r + 1][c + 1] : load_px<F32>(im, x, y, unused);
+        if (A.flags) {
+            const uint8_t f = rep ? 1 : 0;
+            A.flags[i] = A.keep ? (uint8_t)(A.flags[i] | f) : f;
+        }
+        if (rep) atomicAdd(&nrep, 1);
+    }
+    __syncthreads();
+    if (t == 0 && A.count && nrep) atomicAdd(A.count, nrep);
+}
+
 cudaError_t launch_cr(const Image& im, float gain, float rn, float sigclip, float objlim, float* out, uint8_t* flags,
                       int* count, cudaStream_t st)
 {
@@ -660,17 +723,33 @@ cudaError_t launch_cr(const Image& im, float gain, float rn, float sigclip, floa
     return cudaGetLastError();
 }
 
+// Most pixels of a frame for the block form and for 2 rows a warp in place of 8
+// (fewer rows read and sort more halo rows, but spread a small frame over more
+// warps).  Blocks, 2 rows and 8 rows: 512 x 512 27, 45, 69 us; 1 MP 33, 36,
+// 49; 2 MP 43, 46, 55; 4 MP 61, 51, 58; 12 MP 130, 109, 90; 17 MP 172, 138, 112.
+constexpr int64_t RTN_BLOCK_PIXELS = 2 << 20, RTN_FEW_PIXELS = 6 << 20;
+
 cudaError_t launch_rtn(const Image& im, float thr, float* out, uint8_t* flags, bool keep, int* count,
                        cudaStream_t st)
 {
     RtnArgs A;
     A.im = im; A.t = thr; A.out = out; A.flags = flags; A.keep = keep ? 1 : 0; A.count = count;
-    const int64_t warps = (int64_t)((im.W + 127) / 128) * ((im.H + RTN_ROWS - 1) / RTN_ROWS);
-    const int blocks = (int)((warps + RTN_NT / 32 - 1) / (RTN_NT / 32));
+    const int64_t pixels = (int64_t)im.W * im.H;
+    if (pixels <= RTN_BLOCK_PIXELS && im.H <= 65535 * CM_B) {     // (a grid is 65,535 blocks high)
+        const dim3 g((im.W + CM_B - 1) / CM_B, (im.H + CM_B - 1) / CM_B);
+        if (im.is_f32) k_rtn_block<true, false><<<g, CM_NT, 0, st>>>(A);
+        else if (im.mask) k_rtn_block<false, false><<<g, CM_NT, 0, st>>>(A);
+        else k_rtn_block<false, true><<<g, CM_NT, 0, st>>>(A);
+        return cudaGetLastError();
+    }
     const bool vec = (im.pitch & 3) == 0 && (((uintptr_t)im.data) & (im.is_f32 ? 15 : 7)) == 0;
     const bool ovec = (im.W & 3) == 0 && (((uintptr_t)out) & 15) == 0 && (((uintptr_t)flags) & 3) == 0;
-    if (im.is_f32) k_rtn<true><<<blocks, RTN_NT, 0, st>>>(A, vec, ovec);
-    else k_rtn<false><<<blocks, RTN_NT, 0, st>>>(A, vec, ovec);
+    auto run = [&](auto kern, int rows) {
+        const int64_t warps = (int64_t)((im.W + 127) / 128) * ((im.H + rows - 1) / rows);
+        kern<<<(int)((warps + RTN_NT / 32 - 1) / (RTN_NT / 32)), RTN_NT, 0, st>>>(A, vec, ovec);
+    };
+    if (pixels <= RTN_FEW_PIXELS) im.is_f32 ? run(k_rtn<true, 2>, 2) : run(k_rtn<false, 2>, 2);
+    else im.is_f32 ? run(k_rtn<true, 8>, 8) : run(k_rtn<false, 8>, 8);
     return cudaGetLastError();
 }
 
