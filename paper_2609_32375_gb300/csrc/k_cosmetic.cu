@@ -453,6 +453,16 @@ __device__ __forceinline__ float med3_nan(float a, float b, float c)
     return max_nan(min_nan(a, b), min_nan(max_nan(a, b), c));
 }
 
+// the median of a window with bad pixels (out of line: it stands in the middle
+// of k_rtn's row loop, four times)
+struct Window {
+    float v[9];
+};
+__device__ __noinline__ float median_bad(Window w)
+{
+    return median_net<9, 16>(w.v);
+}
+
 // A warp takes 128 columns, a lane 4 of them, over ROWS rows, with the
 // medians of 3 along three rows in registers; neighbours' columns come by
 // shuffle.  The window's median lies between the smallest and the largest of
@@ -571,19 +581,16 @@ __global__ void __launch_bounds__(RTN_NT) k_rtn(const __grid_constant__ RtnArgs 
             const bool maybe = !(max_nan(o[e] - lo, hi - o[e]) <= A.t) && x0 + e < W;
             if (!__any_sync(0xffffffffu, maybe)) continue;
             if (maybe) {
-                float v[9] = {up.w[e], up.w[e + 1], up.w[e + 2], mid.w[e], mid.w[e + 1], mid.w[e + 2],
-                              down.w[e], down.w[e + 1], down.w[e + 2]};
+                Window w = {up.w[e], up.w[e + 1], up.w[e + 2], mid.w[e], mid.w[e + 1], mid.w[e + 2],
+                            down.w[e], down.w[e + 1], down.w[e + 2]};
+                const float x = mid.w[e + 1];                // NaN where the pixel is bad
                 bool bad = false;
                 if (F32 || im.mask) {
 #pragma unroll
-                    for (int k = 0; k < 9; ++k) bad = bad || isnan(v[k]);
+                    for (int k = 0; k < 9; ++k) bad = bad || isnan(w.v[k]);
                 }
-                if (bad) {
-                    if (outlier(x0 + e, y, &med[e])) hits |= 1u << e;
-                } else {
-                    med[e] = med_sel<9>(v);
-                    if (fabsf(o[e] - med[e]) > A.t) hits |= 1u << e;
-                }
+                med[e] = bad ? median_bad(w) : med_sel<9>(w.v);
+                if (!isnan(x) && fabsf(x - med[e]) > A.t) hits |= 1u << e;      // NaN comparisons are false
             }
         }
         // an outlier is replaced when none of its neighbours is one
