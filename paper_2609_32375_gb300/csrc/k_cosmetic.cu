@@ -86,29 +86,26 @@ __device__ __forceinline__ void sort_net(float (&v)[P])
     OESort<0, P, P>::run(v);
 }
 
-// median of the non-NaN values among the N values in (NaN when none; the
-// mean of the two middle values for an even count): NaN sorts last as +inf
+// median of the non-NaN values among the N values in (N odd; NaN when none;
+// the mean of the two middle values for an even count).  NaNs become +inf and
+// -inf in turn, so that the middle values stand at fixed places: at places that
+// follow from the count, the sorted values went through local memory.
 template <int N, int P>
 __device__ __forceinline__ float median_net(const float (&in)[N])
 {
+    static_assert(N % 2 == 1 && N < P, "an odd window, padded to a power of two");
     float v[P];
-    int k = 0;
+    unsigned bad = 0;
 #pragma unroll
     for (int i = 0; i < P; ++i) {
-        const float x = i < N ? in[i] : NAN;
+        const float x = i < N ? in[i] : INFINITY;
         const bool ok = !isnan(x);
-        v[i] = ok ? x : INFINITY;
-        k += ok ? 1 : 0;
+        v[i] = ok ? x : __uint_as_float(0x7f800000u | bad << 31);
+        bad += ok ? 0u : 1u;
     }
     sort_net<P>(v);
-    const int h = k / 2;
-    float a = 0.f, b = 0.f;
-#pragma unroll
-    for (int j = 0; j < N; ++j) {
-        a = j == h ? v[j] : a;
-        b = j == h - 1 ? v[j] : b;
-    }
-    return k == 0 ? NAN : ((k & 1) ? a : 0.5f * (a + b));
+    const float a = v[N / 2], b = v[N / 2 - 1];
+    return bad == N ? NAN : ((bad & 1u) ? 0.5f * (a + b) : a);
 }
 
 template <bool F32>
@@ -324,7 +321,7 @@ __device__ __forceinline__ void cr_flags_clean(CrBlock& s, CrMaps& M, const CrAr
 // each CTA looks whether its part does.  17 MP uint16: 804 us with every
 // map computed at every pixel, 184 us so.
 template <bool F32, bool CLEAN>
-__global__ void __launch_bounds__(CM_NT, CLEAN ? 5 : 2) k_cr(const __grid_constant__ CrArgs A)
+__global__ void __launch_bounds__(CM_NT, CLEAN ? 5 : 3) k_cr(const __grid_constant__ CrArgs A)
 {
     __shared__ CrBlock s;
     __shared__ CrMaps maps;
