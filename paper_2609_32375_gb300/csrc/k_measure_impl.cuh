@@ -116,6 +116,20 @@ __device__ __forceinline__ float pixel_area(float dx0, float dy0, float r)
 // once per row for whichever lanes meet the circle.
 constexpr int QCAP = 64;      // at most 31 waiting + 32 added by one row
 constexpr int MEAS_NT = 256;
+// CTAs an SM holds for nr radii: the sums of six radii and more do not fit the
+// registers of three (15,000 positions, radii up to 15: six radii 404 us with
+// three CTAs and 314 with two, eight 688 and 393; three radii 235 and 225, but
+// 2,500 positions with them 65 and 69)
+constexpr int meas_ctas(int nr) { return nr > 5 ? 2 : 3; }
+// The kernels are compiled for 0 to 6 and 8 radii; 7 take the last, whose eighth
+// radius is 0 and meets no pixel (an instance of its own came out at 1,138 us for
+// those positions).  nr: the radii in the results.
+template <int NR>
+__device__ __forceinline__ int meas_nr(const ApSpec& ap)
+{
+    if constexpr (NR == MAX_NR) return ap.nr;
+    else return NR;
+}
 
 // a row's terms, each computed by one lane: the y-spline's coefficients in
 // pairs (for the background and the noise at once), ny^2 and the larger
@@ -377,11 +391,12 @@ __device__ void aperture_warp(const Image& im, const SplineTab& sb, const Spline
     const DF s = df_reduce_scatter<NV>(acc);
     const int idx = scatter_index<NV>(lane);
     const bool first = (lane & ((32 / NV) - 1)) == 0;     // one writer per value
-    if (first && idx < NR) {
+    const int nr = meas_nr<NR>(ap);
+    if (first && idx < nr) {
         reinterpret_cast<float2*>(flux)[idx] = make_float2(s.hi, s.lo);
         aflags[idx] = ((pk >> idx) & 1u ? GP_FLAG_BAD : 0u) | ((pk >> (8 + idx)) & 1u ? GP_FLAG_SAT : 0u);
     }
-    if (first && idx >= NRA && idx < NRA + NR) reinterpret_cast<float2*>(ferr)[idx - NRA] = make_float2(s.hi, s.lo);
+    if (first && idx >= NRA && idx < NRA + nr) reinterpret_cast<float2*>(ferr)[idx - NRA] = make_float2(s.hi, s.lo);
 }
 
 // Radius k's results at (cx, cy) from the raw sums in *flux and *ferr: the
@@ -427,7 +442,7 @@ __device__ __forceinline__ const MeasureArgs& measure_frame(const MeasureArgs* _
 }
 
 template <bool F32, int NR, bool BATCH>
-__global__ void __launch_bounds__(MEAS_NT, 3) k_measure(const MeasureArgs* __restrict__ batch,
+__global__ void __launch_bounds__(MEAS_NT, meas_ctas(NR)) k_measure(const MeasureArgs* __restrict__ batch,
                                                      const __grid_constant__ MeasureArgs one)
 {
     pdl_wait();
@@ -438,17 +453,17 @@ __global__ void __launch_bounds__(MEAS_NT, 3) k_measure(const MeasureArgs* __res
     const int wid = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int nw = (gridDim.x * blockDim.x) >> 5;
     const int ncomp = min(*A.C.count, A.C.cap);
-    const int nrow = min(ncomp, A.capacity);
+    const int nrow = min(ncomp, A.capacity), nr = meas_nr<NR>(A.ap);
     for (int r = wid; r < nrow; r += nw) {
         const double2 xy = A.C.xy[A.C.perm[r]];
         if constexpr (NR > 0)
-            aperture_warp<F32, NR>(A.im, A.sb, A.sr, A.ap, xy.x, xy.y, A.apflux + (int64_t)r * NR,
-                                   A.apferr + (int64_t)r * NR, A.apflags + (int64_t)r * NR, wq);
+            aperture_warp<F32, NR>(A.im, A.sb, A.sr, A.ap, xy.x, xy.y, A.apflux + (int64_t)r * nr,
+                                   A.apferr + (int64_t)r * nr, A.apflags + (int64_t)r * nr, wq);
     }
 }
 
 template <bool F32, int NR>
-__global__ void __launch_bounds__(MEAS_NT, 3) k_aperture(Image im, SplineTab sb, SplineTab sr,
+__global__ void __launch_bounds__(MEAS_NT, meas_ctas(NR)) k_aperture(Image im, SplineTab sb, SplineTab sr,
                                                       const __grid_constant__ ApSpec ap,
                                                       const double* xs, const double* ys, int n, double* flux,
                                                       double* ferr, uint32_t* fl)
@@ -456,10 +471,10 @@ __global__ void __launch_bounds__(MEAS_NT, 3) k_aperture(Image im, SplineTab sb,
     __shared__ ApWarp warps[MEAS_NT / 32];
     ApWarp* wq = warps + (threadIdx.x >> 5);
     const int wid = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int nw = (gridDim.x * blockDim.x) >> 5;
+    const int nw = (gridDim.x * blockDim.x) >> 5, nr = meas_nr<NR>(ap);
     for (int i = wid; i < n; i += nw)
-        aperture_warp<F32, NR>(im, sb, sr, ap, xs[i], ys[i], flux + (int64_t)i * NR, ferr + (int64_t)i * NR,
-                               fl + (int64_t)i * NR, wq);
+        aperture_warp<F32, NR>(im, sb, sr, ap, xs[i], ys[i], flux + (int64_t)i * nr, ferr + (int64_t)i * nr,
+                               fl + (int64_t)i * nr, wq);
 }
 
 // The catalog rows in label order: thread (row, 0) copies the segment's
@@ -525,8 +540,7 @@ static cudaError_t dispatch_nr(int nr, Args... args)
     case 4: return Launch<F32, 4>::run(args...);
     case 5: return Launch<F32, 5>::run(args...);
     case 6: return Launch<F32, 6>::run(args...);
-    case 7: return Launch<F32, 7>::run(args...);
-    default: return Launch<F32, 8>::run(args...);
+    default: return Launch<F32, MAX_NR>::run(args...);
     }
 }
 
