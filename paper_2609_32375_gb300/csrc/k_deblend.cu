@@ -18,7 +18,7 @@
 //    first pixels); the objects are labelled 1 + their minimum linear index.
 //
 // A team of threads per candidate segment, its bounding box in global
-// scratch: a warp for boxes up to DB_SMALL pixels, a group of DB_GW warps up to
+// scratch: a warp for boxes up to DB_SMALL pixels (more in crowded frames), a group of DB_GW warps up to
 // DB_MED, a CTA above, a cluster of 8 CTAs above DB_BIG.  One launch serves all:
 // its clusters first work through the big candidates together, then each CTA
 // through the larger ones, each group through the middle ones and each warp
@@ -27,7 +27,9 @@
 // pixels takes 30 levels of five passes over its pixels, then some 250 growth
 // rounds, 0.96 ms in all (a single CTA took 6 to 15 ms on such a field).  The
 // thousands of stars beside it are short and wait on memory and barriers, so
-// many run side by side.  17 MP dense fields: 11.4 ms a call before, 1.9 now.
+// many run side by side.  It hangs on the field: two crowded 17 MP frames with
+// nebulosity 11.4 and 11.5 ms a call with a CTA a candidate, 1.9 and 1.7 so; the
+// 151 MP frame 19.0 and 3.4; a 4 MP CCD frame without nebulosity 0.92 and 0.60.
 //
 // Sums of m are exact 64-bit fixed-point integers (m scaled by 2^20), the
 // level sets' components come from a lock-free union-find whose roots are the
@@ -60,9 +62,16 @@ constexpr int DB_CL = 8;                     // CTAs of a cluster
 // in place of the groups 0.59, but then a crowded 17 MP field, whose groups
 // number thousands, 5 % more.  64 against 128: the 162 stars of a 512 x 512 frame
 // with boxes up to 100 pixels 0.30 and 0.38 ms.
+// DB_BIG at 4,096 or 16,384 makes no difference to a crowded 17 MP field.
 constexpr int DB_SMALL = 64, DB_MED = 1024, DB_BIG = 8192;
+// a warp's most in frames with more segments than the chip has warps, where
+// throughput counts (the 40,130 of a crowded 151 MP frame, 6,000 of them with
+// boxes of 65 to 128 pixels: 3.74 ms with 64, 3.43 with 128, 3.37 with 256)
+constexpr int DB_MANY = 32 * 152, DB_SMALL_MANY = 128;
 constexpr int DB_GW = 8;                     // warps of a group
-constexpr int DB_ROW = 1024;                 // box pixels of an object's catalog row: a warp's most
+// box pixels of an object's catalog row: a warp's most (crowded 17 MP field, 256,
+// 1,024 and 4,096: 1.91, 1.91 and 1.96 ms)
+constexpr int DB_ROW = 1024;
 // the call's counters, one 256-byte block cleared per call: candidates larger
 // than DB_SMALL, staged objects, small candidates, big ones; the next big,
 // CTA's, small and group's one to claim; then the first big candidates' indexes
@@ -461,7 +470,9 @@ __device__ __forceinline__ void db_emit(const DeblendArgs& A, const DbSums& v, u
 }
 
 // ------------------------------------------------------------ a segment ---
-constexpr int DB_TREE_ONE = 2048;    // active pixels that one CTA of a cluster works on alone
+// active pixels that one CTA of a cluster works on alone (crowded 17 MP field,
+// 512, 2,048 and 8,192: 1.91, 1.91 and 1.97 ms)
+constexpr int DB_TREE_ONE = 2048;
 
 // the branch tree from level i on, over the list lst of the nl pixels still
 // active, down to a list of `least`
@@ -1094,10 +1105,11 @@ __global__ void __launch_bounds__(256) k_db_select(const int* __restrict__ n_dev
                                                    int* cand, int* ctl, int64_t* bytes)
 {
     const int n = min(*n_dev, cap);
+    const int warps_most = n > DB_MANY ? DB_SMALL_MANY : DB_SMALL;
     for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < n; r += gridDim.x * blockDim.x) {
         if (npix[r] < 2 * minarea) continue;
         const int64_t w = xmax[r] - xmin[r] + 1, h = ymax[r] - ymin[r] + 1;
-        const bool small = w * h <= DB_SMALL;
+        const bool small = w * h <= warps_most;
         const int i = atomicAdd(ctl + (small ? DBC_SMALL : DBC_N), 1);
         const int k = small ? cap - 1 - i : i;
         if (w * h > DB_BIG) {

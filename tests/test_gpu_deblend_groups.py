@@ -60,3 +60,31 @@ def test_box_sizes_around_the_teams(copies, f32):
     for k in ("label", "npix", "xmin", "xmax", "ymin", "ymax", "xpeak", "ypeak", "flags"):
         assert np.array_equal(cat[k], rc[k]), k
     assert np.array_equal(cat["flux_iso"], rc["flux"])       # sums of whole numbers
+
+
+def test_more_segments_than_the_chip_has_warps():
+    """Where warps take larger boxes: every rectangle splits as its like does in a small frame."""
+    def patches(copies):
+        a = field(copies).astype(np.uint16)
+        H, W = a.shape
+        kern, mesh = np.ones((1, 1), np.float32), 128
+        my, mx = -(-H // mesh), -(-W // mesh)
+        ctx = gp.Context(0, workspace_bytes=1 << 30)
+        t = torch.from_numpy(a).cuda()
+        bkg = {"bkg_mesh": torch.full((my, mx), 1000.0, device="cuda"),
+               "rms_mesh": torch.full((my, mx), 30.0, device="cuda"), "mesh": mesh}
+        det = ctx.gp_detect(t, bkg, kern, 1.5, 5, 20000)
+        seg = det["segmap"].clone()
+        db = ctx.gp_deblend(t, bkg, kern, 1.5, 5, seg, det["catalog"])
+        ctx.sync()
+        n = copies * len(BOXES)
+        assert int(det["catalog"]["n"].item()) == n and db["counts"].cpu().numpy().tolist() == [n, 2 * n]
+        s, nx = seg.cpu().numpy(), int(np.ceil(np.sqrt(n)))
+        for i in range(n):
+            (h, w), y, x = BOXES[i % len(BOXES)], 1 + 44 * (i // nx), 1 + 44 * (i % nx)
+            yield i, np.unique(s[y:y + h, x:x + w], return_inverse=True)[1].reshape(-1)
+
+    like = {i % 63: p for i, p in patches(9)}                # 9 boxes by 7 levels
+    assert len(like) == 63
+    for i, p in patches(600):
+        assert np.array_equal(p, like[i % 63]), i
