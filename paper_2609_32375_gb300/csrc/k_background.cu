@@ -479,7 +479,10 @@ __device__ void boxstats_u16_box(const BoxArgs& A, int box, uint32_t* hist)
 // Threads a box by the number of boxes: 128 keep 8 boxes an SM in flight; a
 // frame with fewer boxes than that takes 256 or 512, as it lasts as long as
 // one box (256 boxes of 128 x 128: 31 us with 128 threads, 26 with 512; 512
-// boxes of 256 x 256: 51 us with 128 threads, 56 with 512, 39 with 256).
+// boxes of 256 x 256: 51 us with 128 threads, 56 with 512, 39 with 256).  Boxes
+// of fewer than 32 values a thread keep the smaller CTAs: 576 to 1,024 boxes of
+// 64 x 64 take 27 to 31 us with 128 threads, 27 to 39 with 256 or 512 (a handful
+// of them 25 and 23, of 90 x 90 31 and 24).
 constexpr int NWIN = 4096;
 constexpr int NOUT = 1024;              // values outside the window a box may list
 constexpr int WCB = 64;                 // values per coarse bin of the window
@@ -896,8 +899,8 @@ __global__ void __launch_bounds__(WB_NT, 1024 / WB_NT) k_boxstats_win(const BoxA
 //              warp 0: mean; the median's bin              | barrier
 //              squared deviations; that bin's values       | barrier
 //              warp 0: sigma, median, next range           | barrier
-// Bound by instruction issue and the barriers' latency: 32 us for the 256 boxes
-// of a 1 MP frame at mesh 64 and 106 us for a masked 9 MP one, where a bitonic
+// Bound by instruction issue and the barriers' latency: 34 us for the 256 boxes
+// of a 1 MP frame at mesh 64 and 111 us for a masked 9 MP one, where a bitonic
 // sort of each box (78 block-wide steps of 4,096 values) took 183 and 721; the
 // quantiles of a 17 MP frame take 91 us against 523.  Two float32 values take one paired operation
 // in the compensated sums.  The box's mean and sigma are float64; a pass takes

@@ -261,10 +261,11 @@ __device__ __forceinline__ bool cr_decide(const CrBlock& s, const CrArgs& A, int
 }
 
 // a block without one: candidates by the bound on S, then a warp for each.
-// Bound by instruction issue and the barriers around the few candidates: the
-// staging and the bound's own arithmetic take about 15 instructions a pixel,
-// a candidate some 700, the full maps 19,000 a block; so more than CR_MOST
-// candidates take those.
+// Bound by latency: the staging and the bound take some 600 warp instructions a
+// block, but the eight warps meet at barriers, and between two of them one or two
+// decide a candidate by 25- and 49-value rank counts, one shuffle after
+// another, while the others wait.  A candidate is some 700 instructions, the
+// full maps 19,000 a block; so more than CR_MOST candidates take those.
 constexpr int CR_MOST = 28;
 
 __device__ __forceinline__ void cr_flags_clean(CrBlock& s, CrMaps& M, const CrArgs& A)
@@ -319,7 +320,9 @@ __device__ __forceinline__ void cr_flags_clean(CrBlock& s, CrMaps& M, const CrAr
 
 // CLEAN: the frame cannot hold a bad pixel (uint16 without a mask); else
 // each CTA looks whether its part does.  17 MP uint16: 804 us with every
-// map computed at every pixel, 184 us so.
+// map computed at every pixel, 175 us so.  12 MP with one pixel in 500 masked, so
+// that most blocks take the whole maps: 7.0 ms with the middle value picked from
+// local memory, 0.86 so (median_net).
 template <bool F32, bool CLEAN>
 __global__ void __launch_bounds__(CM_NT, CLEAN ? 5 : 3) k_cr(const __grid_constant__ CrArgs A)
 {
@@ -467,8 +470,9 @@ __device__ __noinline__ float median_bad(Window w)
 // only a pixel more than t from one of those, or with a bad pixel in its
 // window (NaN), can be an outlier.  Those take the median of the 9 values in
 // registers; an outlier's 8 neighbours are then tested by 8 lanes, or by its
-// own lane where a row holds many (a track).  Bound by the row loop's latency.  17 MP after the cosmic-ray filter: 153 us with the median
-// taken at every pixel of 32 x 32 blocks in shared memory, 87 us so.
+// own lane where a row holds many (a track).  Bound by the row loop's latency.
+// 17 MP after the cosmic-ray filter: 153 us with the median taken at every pixel
+// of 32 x 32 blocks in shared memory, 75 us so.
 constexpr int RTN_NT = 64;
 // lanes with outliers in a row: up to this many, the warp's lanes test one's
 // neighbours together, a round trip each; more (a track along the row) and each
@@ -730,7 +734,8 @@ cudaError_t launch_cr(const Image& im, float gain, float rn, float sigclip, floa
 // Most pixels of a frame for the block form and for 2 rows a warp in place of 8
 // (fewer rows read and sort more halo rows, but spread a small frame over more
 // warps).  Blocks, 2 rows and 8 rows: 512 x 512 27, 45, 69 us; 1 MP 33, 36,
-// 49; 2 MP 43, 46, 55; 4 MP 61, 51, 58; 12 MP 130, 109, 90; 17 MP 172, 138, 112.
+// 49; 2 MP 43, 46, 55; 4 MP 61, 51, 58; 12 MP 130, 109, 90; 17 MP 172, 138, 112
+// (with windows that hold a bad pixel read again, which the last two no longer do).
 constexpr int64_t RTN_BLOCK_PIXELS = 2 << 20, RTN_FEW_PIXELS = 6 << 20;
 
 cudaError_t launch_rtn(const Image& im, float thr, float* out, uint8_t* flags, bool keep, int* count,

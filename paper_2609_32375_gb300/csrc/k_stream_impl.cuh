@@ -36,7 +36,7 @@
 //           mirrored coordinates found once), two groups ahead in registers.
 //           A mask is read in the same way: a masked float becomes NaN in
 //           the stage, a masked uint16 a bit in a register.  A masked 9 MP
-//           float32 frame with unaligned rows takes 118 us (350 with each
+//           float32 frame with unaligned rows takes 104 us (350 with each
 //           element and mask byte loaded, at coordinates mirrored by integer
 //           division, where it was used).
 // Batches whose frames all allow tensor maps use them too: eight 4 MP uint16
